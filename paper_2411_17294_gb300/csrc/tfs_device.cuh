@@ -73,6 +73,15 @@ __device__ __forceinline__ void assemble_M(const double K[3][3], double a, doubl
     });
 }
 
+// |a| > |b| on the integer pipe (the FP64 pipe is what the FP64 solves wait
+// for): the bit patterns of magnitudes order as the values do; false for a NaN
+// on either side, as the comparison of the values is.
+__device__ __forceinline__ bool abs_greater(double a, double b) {
+    const unsigned long long ia = (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
+    const unsigned long long ib = (unsigned long long)__double_as_longlong(b) & 0x7fffffffffffffffull;
+    return ia > ib && ia <= 0x7ff0000000000000ull;
+}
+
 // In-place Gaussian elimination with partial pivoting on a small dense system.
 // Pivot search by compare-and-swap (no dynamic register indexing): the largest
 // |entry| of column k among rows k.. ends up in row k, ties keep the earlier row.
@@ -84,7 +93,7 @@ __device__ __forceinline__ bool gauss_pp(double M[NC][NC], double x[NC], double 
         constexpr int k = decltype(kk)::value;
         static_for<k + 1, NC>([&](auto ii) {
             constexpr int i = decltype(ii)::value;
-            const bool sw = fabs(M[i][k]) > fabs(M[k][k]);
+            const bool sw = abs_greater(M[i][k], M[k][k]);
             static_for<k, NC>([&](auto jj) {
                 constexpr int j = decltype(jj)::value;
                 const double t0 = M[k][j], t1 = M[i][j];
@@ -131,7 +140,7 @@ __device__ __forceinline__ bool gauss_pp_multi(double M[NC][NC], double X[NC][NR
         constexpr int k = decltype(kk)::value;
         static_for<k + 1, NC>([&](auto ii) {
             constexpr int i = decltype(ii)::value;
-            const bool sw = fabs(M[i][k]) > fabs(M[k][k]);
+            const bool sw = abs_greater(M[i][k], M[k][k]);
             static_for<k, NC>([&](auto jj) {
                 constexpr int j = decltype(jj)::value;
                 const double t0 = M[k][j], t1 = M[i][j];

@@ -1,4 +1,6 @@
-// Forward stress step: one launch advances every grid point from t_n to t_{n+1}.
+// Forward stress step in FP32 storage: one launch advances every grid point from
+// t_n to t_{n+1} (FP64 storage: tfs_forward64.cu, whose paper's variable takes
+// its transport pre-pass from here).
 //
 // Per point (Section 4.1 with the kernel compression of Section 2.2):
 //   kappa* = 2 kappa^n - kappa^{n-1}, E = 2 sigma^n - sigma^{n-1}
@@ -27,19 +29,17 @@
 // (94% of the bytes) and every per-point input are in flight without holding
 // registers, and the compute phase makes no global loads.  Inside a tile,
 // warp w handles stress components w and w + 3 in 3D (w in 2D), lane = point:
-// it forms Q_j = b1 x + b2 y from shared memory, the history sum H (FP32
-// storage: Kahan summation of terms formed exactly by FMA, eta_j split
-// hi + lo) and its components of the right-hand side.  Warp 0 then solves the
-// 32 point systems with lane = point; all warps write the new mode level from
-// the Q_j with streaming stores.  Every mode value is read once and written
-// once.
+// it forms Q_j = b1 x + b2 y from shared memory, the history sum H (Kahan
+// summation of terms formed exactly by FMA, eta_j split hi + lo) and its
+// components of the right-hand side.  Warp 0 then solves the 32 point systems
+// with lane = point; all warps write the new mode level from the Q_j with
+// streaming stores.  Every mode value is read once and written once.
 //
-// Point solve.  FP64 storage: FP64 Gaussian elimination with partial
-// pivoting.  FP32 storage: FP32 LU with partial pivoting, one refinement step
-// whose residual R - M x0 is evaluated in double-float arithmetic (TwoSum /
-// TwoProd, ~44-bit), correction through the same factors: the solution of the
-// system as given is accurate far beyond the FP32 rounding of the stored
-// result, and the FP64 pipe (1/64 of the FP32 rate on this GPU) stays free.
+// Point solve.  FP32 LU with partial pivoting, one refinement step whose
+// residual R - M x0 is evaluated in double-float arithmetic (TwoSum / TwoProd,
+// ~44-bit), correction through the same factors: the solution of the system as
+// given is accurate far beyond the FP32 rounding of the stored result, and the
+// FP64 pipe (1/64 of the FP32 rate on this GPU) stays free.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -848,8 +848,7 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
     constexpr int NC = Packed<DIM>::NC;
     constexpr int W = StepShape<DIM>::W;
     constexpr int CPW = StepShape<DIM>::CPW;
-    constexpr bool F32 = sizeof(T) == 4;
-    static_assert(!QR || F32, "the register variant serves FP32 storage");
+    static_assert(sizeof(T) == 4, "FP64 storage: tfs_forward64.cu");
     float qr[QR ? CPW : 1][QR ? kQR : 1];   // Q_j in registers (QR)
     const int lane = threadIdx.x;
     const int w = threadIdx.y;
@@ -861,13 +860,11 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
 
     // ---- (a4) history sums over the modes of this thread's components
     //      (Q_j stored in place of level n-1)
-    double Hd[CPW];
     f2 Hf[CPW];
     T s0c[CPW];
 #pragma unroll
     for (int cc = 0; cc < CPW; ++cc) {
         const int c = w + cc * W;
-        Hd[cc] = 0.0;
         Hf[cc] = f2{0.0f, 0.0f};
         s0c[cc] = has_s0 ? buf[(S.s0 + c) * kTile + lane] : (T)0;
     }
@@ -877,18 +874,14 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
             const int c = w + cc * W;
             const T sn = buf[(S.sig + c) * kTile + lane];
             const T sm = buf[(S.sig + NC + c) * kTile + lane];
-            if constexpr (F32) {
-                // b1 sigma^n + b2 sigma^{n-1} + b0 sigma0: exact products by powers of two, TwoProd for b0
-                const f2 h = two_sum_f2(-2.0f * (float)sn, 0.5f * (float)sm);
-                Hf[cc] = f2_add(h, two_prod(1.5f, (float)s0c[cc]));
-            } else {
-                Hd[cc] = kB1 * (double)sn + kB2 * (double)sm + kB0 * (double)s0c[cc];
-            }
+            // b1 sigma^n + b2 sigma^{n-1} + b0 sigma0: exact products by powers of two, TwoProd for b0
+            const f2 h = two_sum_f2(-2.0f * (float)sn, 0.5f * (float)sm);
+            Hf[cc] = f2_add(h, two_prod(1.5f, (float)s0c[cc]));
         }
     } else {
         const T* lv0 = buf + (w * kTile + lane);
         T* lv1 = buf + ((m * NC + w) * kTile + lane);
-        if constexpr (F32 && COMP) {
+        if constexpr (COMP) {
             // Kahan summation of the terms eta_j Q_j: each term enters as
             // fma(eta_hi, Q, fma(eta_lo, Q, -comp)) -- the product is exact inside
             // the FMA, so the term is rounded once -- and the rounding error of
@@ -931,7 +924,7 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
             }
 #pragma unroll
             for (int cc = 0; cc < CPW; ++cc) Hf[cc] = fast_two_sum(hs[cc], -comp[cc]);
-        } else if constexpr (F32) {
+        } else {
             float hs[CPW];
 #pragma unroll
             for (int cc = 0; cc < CPW; ++cc) hs[cc] = 0.0f;
@@ -962,17 +955,6 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
             }
 #pragma unroll
             for (int cc = 0; cc < CPW; ++cc) Hf[cc] = f2_from(hs[cc]);
-        } else {
-#pragma unroll 2
-            for (int j = 0; j < m; ++j) {
-#pragma unroll
-                for (int cc = 0; cc < CPW; ++cc) {
-                    const int o = (j * NC + cc * W) * kTile;
-                    const double qj = kB1 * (double)lv0[o] + kB2 * (double)lv1[o];
-                    lv1[o] = (T)qj;
-                    Hd[cc] = fma(A.mc.eta[j], qj, Hd[cc]);
-                }
-            }
         }
     }
 
@@ -982,8 +964,7 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
 #pragma unroll
     for (int cc = 0; cc < CPW && PAPER; ++cc) {
         const int c = w + cc * W;
-        if constexpr (F32) reinterpret_cast<f2*>(sR_raw)[c * kTile + lane] = Hf[cc];
-        else reinterpret_cast<double*>(sR_raw)[c * kTile + lane] = Hd[cc];
+        reinterpret_cast<f2*>(sR_raw)[c * kTile + lane] = Hf[cc];
     }
 #pragma unroll
     for (int cc = 0; cc < CPW && !PAPER; ++cc) {
@@ -993,21 +974,14 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
         const T km_ij = buf[(S.km + ci * DIM + cj) * kTile + lane];
         const T kn_ji = buf[(S.kn + cj * DIM + ci) * kTile + lane];
         const T km_ji = buf[(S.km + cj * DIM + ci) * kTile + lane];
-        if constexpr (F32) {
-            const f2 kab = two_sum_f2(2.0f * (float)kn_ij, -(float)km_ij);
-            const f2 kba = two_sum_f2(2.0f * (float)kn_ji, -(float)km_ji);
-            const f2 ks = f2_add(kab, kba);
-            const f2 eta{A.eta_f2.hi, A.eta_f2.lo}, src{A.src_f2.hi, A.src_f2.lo};
-            f2 R = f2_add(f2_mul_f(eta, (float)s0c[cc]), f2_neg(Hf[cc]));
-            R = f2_add(R, f2_mul(src, ks));
-            if constexpr (TRANSPORT) R = f2_add_f(R, -(float)buf[(S.tr + c) * kTile + lane]);
-            reinterpret_cast<f2*>(sR_raw)[c * kTile + lane] = R;
-        } else {
-            const double ks = (2.0 * (double)kn_ij - (double)km_ij) + (2.0 * (double)kn_ji - (double)km_ji);
-            double R = A.eta * (double)s0c[cc] - Hd[cc] + A.dt * A.G * A.g * ks;
-            if constexpr (TRANSPORT) R -= (double)buf[(S.tr + c) * kTile + lane];
-            reinterpret_cast<double*>(sR_raw)[c * kTile + lane] = R;
-        }
+        const f2 kab = two_sum_f2(2.0f * (float)kn_ij, -(float)km_ij);
+        const f2 kba = two_sum_f2(2.0f * (float)kn_ji, -(float)km_ji);
+        const f2 ks = f2_add(kab, kba);
+        const f2 eta{A.eta_f2.hi, A.eta_f2.lo}, src{A.src_f2.hi, A.src_f2.lo};
+        f2 R = f2_add(f2_mul_f(eta, (float)s0c[cc]), f2_neg(Hf[cc]));
+        R = f2_add(R, f2_mul(src, ks));
+        if constexpr (TRANSPORT) R = f2_add_f(R, -(float)buf[(S.tr + c) * kTile + lane]);
+        reinterpret_cast<f2*>(sR_raw)[c * kTile + lane] = R;
     }
     // QR: the solving warp's stage inputs in registers, so that the hook may
     // refill the whole stage
@@ -1062,83 +1036,46 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
             //     = -b1 Phi^n - b2 Phi^{n-1} + dt (L(kappa*) h - h/Wi) + dt G (kappa* + kappa*^T) Psi0 [- A]
             // (A: the transport of E = 2 Psi^n - Psi^{n-1}, from the pre-pass)
             // Psi^{n+1} = xi Phi^{n+1} + h
-            if constexpr (F32) {
-                f2 K[3][3];
-                float Kf[3][3];
+            f2 K[3][3];
+            float Kf[3][3];
 #pragma unroll
-                for (int a = 0; a < DIM; ++a)
+            for (int a = 0; a < DIM; ++a)
 #pragma unroll
-                    for (int b = 0; b < DIM; ++b) {
-                        K[a][b] = two_sum_f2(2.0f * kn_at(a * DIM + b), -km_at(a * DIM + b));
-                        Kf[a][b] = K[a][b].hi;
-                    }
-                const f2* sH = reinterpret_cast<const f2*>(sR_raw);
-                f2 h[NC], R[NC], x[NC];
-                if constexpr (QR) {
-                    // h is read after the solve (fewer live registers during it)
-#pragma unroll
-                    for (int r = 0; r < NC; ++r) R[r] = reinterpret_cast<const f2*>(sD)[r * kTile + lane];
-                } else {
-                    float Hs[3][3];
-#pragma unroll
-                    for (int r = 0; r < NC; ++r) {
-                        h[r] = sH[r * kTile + lane];
-                        Hs[Packed<DIM>::I(r)][Packed<DIM>::J(r)] = h[r].hi;
-                        Hs[Packed<DIM>::J(r)][Packed<DIM>::I(r)] = h[r].hi;
-                    }
-                    auto Kat = [&](int a, int b) { return K[a][b]; };
-                    auto Hat = [&](int a, int b) { return Hs[a][b]; };
-#pragma unroll
-                    for (int r = 0; r < NC; ++r)
-                        R[r] = paper_rhs_f32<DIM, TRANSPORT>(A, S, reinterpret_cast<const float*>(buf), lane, Kat, Hat,
-                                                             r);
+                for (int b = 0; b < DIM; ++b) {
+                    K[a][b] = two_sum_f2(2.0f * kn_at(a * DIM + b), -km_at(a * DIM + b));
+                    Kf[a][b] = K[a][b].hi;
                 }
-                if (!solve_point_f32<DIM>(K, A.a_f2, A.dtxi_f2, R, x)) fl |= 2u;
-                const f2 xi{A.xi_f2.hi, A.xi_f2.lo};
+            const f2* sH = reinterpret_cast<const f2*>(sR_raw);
+            f2 h[NC], R[NC], x[NC];
+            if constexpr (QR) {
+                // h is read after the solve (fewer live registers during it)
 #pragma unroll
-                for (int r = 0; r < NC; ++r) {
-                    if constexpr (QR) h[r] = sH[r * kTile + lane];
-                    out[r] = (T)(x[r].hi + x[r].lo);
-                    const f2 ps = f2_add(f2_mul(xi, x[r]), h[r]);
-                    psi[r] = (T)(ps.hi + ps.lo);
-                }
+                for (int r = 0; r < NC; ++r) R[r] = reinterpret_cast<const f2*>(sD)[r * kTile + lane];
             } else {
-                double K[3][3], Hs[3][3];
-#pragma unroll
-                for (int a = 0; a < DIM; ++a)
-#pragma unroll
-                    for (int b = 0; b < DIM; ++b)
-                        K[a][b] = 2.0 * (double)buf[(S.kn + a * DIM + b) * kTile + lane] -
-                                  (double)buf[(S.km + a * DIM + b) * kTile + lane];
-                const double* sH = reinterpret_cast<const double*>(sR_raw);
-                double h[NC], x[NC];
+                float Hs[3][3];
 #pragma unroll
                 for (int r = 0; r < NC; ++r) {
                     h[r] = sH[r * kTile + lane];
-                    Hs[Packed<DIM>::I(r)][Packed<DIM>::J(r)] = h[r];
-                    Hs[Packed<DIM>::J(r)][Packed<DIM>::I(r)] = h[r];
+                    Hs[Packed<DIM>::I(r)][Packed<DIM>::J(r)] = h[r].hi;
+                    Hs[Packed<DIM>::J(r)][Packed<DIM>::I(r)] = h[r].hi;
                 }
+                auto Kat = [&](int a, int b) { return K[a][b]; };
+                auto Hat = [&](int a, int b) { return Hs[a][b]; };
 #pragma unroll
-                for (int r = 0; r < NC; ++r) {
-                    const int i = Packed<DIM>::I(r), j = Packed<DIM>::J(r);
-                    double lh = -A.inv_wi * Hs[i][j];
-#pragma unroll
-                    for (int l = 0; l < DIM; ++l) lh = fma(K[i][l], Hs[l][j], fma(Hs[i][l], K[j][l], lh));
-                    const double pn = (double)buf[(S.sig + r) * kTile + lane];
-                    const double pm = (double)buf[(S.sig + NC + r) * kTile + lane];
-                    x[r] = (2.0 * pn - 0.5 * pm) + A.dt * lh + A.dt * A.G * A.g * (K[i][j] + K[j][i]);
-                    if constexpr (TRANSPORT) x[r] -= (double)buf[(S.tr + r) * kTile + lane];
-                }
-                double M[NC][NC];
-                assemble_M<DIM>(K, A.a, A.dt * A.xi, M);
-                if (!gauss_pp<NC>(M, x, 1e-300)) fl |= 2u;
-#pragma unroll
-                for (int r = 0; r < NC; ++r) {
-                    out[r] = (T)x[r];
-                    psi[r] = (T)fma(A.xi, x[r], h[r]);
-                }
+                for (int r = 0; r < NC; ++r)
+                    R[r] = paper_rhs_f32<DIM, TRANSPORT>(A, S, reinterpret_cast<const float*>(buf), lane, Kat, Hat,
+                                                         r);
             }
-        } else if constexpr (F32) {
+            if (!solve_point_f32<DIM>(K, A.a_f2, A.dtxi_f2, R, x)) fl |= 2u;
+            const f2 xi{A.xi_f2.hi, A.xi_f2.lo};
+#pragma unroll
+            for (int r = 0; r < NC; ++r) {
+                if constexpr (QR) h[r] = sH[r * kTile + lane];
+                out[r] = (T)(x[r].hi + x[r].lo);
+                const f2 ps = f2_add(f2_mul(xi, x[r]), h[r]);
+                psi[r] = (T)(ps.hi + ps.lo);
+            }
+        } else {
             f2 K[3][3];
 #pragma unroll
             for (int a = 0; a < DIM; ++a)
@@ -1152,23 +1089,6 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
             if (!solve_point_f32<DIM>(K, A.a_f2, A.dt_f2, R, x)) fl |= 2u;
 #pragma unroll
             for (int r = 0; r < NC; ++r) out[r] = (T)(x[r].hi + x[r].lo);
-        } else {
-            double K[3][3];
-#pragma unroll
-            for (int a = 0; a < DIM; ++a)
-#pragma unroll
-                for (int b = 0; b < DIM; ++b)
-                    K[a][b] = 2.0 * (double)buf[(S.kn + a * DIM + b) * kTile + lane] -
-                              (double)buf[(S.km + a * DIM + b) * kTile + lane];
-            const double* sR = reinterpret_cast<const double*>(sR_raw);
-            double x[NC];
-#pragma unroll
-            for (int r = 0; r < NC; ++r) x[r] = sR[r * kTile + lane];
-            double M[NC][NC];
-            assemble_M<DIM>(K, A.a, A.dt, M);
-            if (!gauss_pp<NC>(M, x, 1e-300)) fl |= 2u;
-#pragma unroll
-            for (int r = 0; r < NC; ++r) out[r] = (T)x[r];
         }
         bool finite = true;
 #pragma unroll
@@ -1178,8 +1098,7 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
             if constexpr (QR) s0r = (T)s0_r[r];
             else s0r = has_s0 ? buf[(S.s0 + r) * kTile + lane] : (T)0;
             // the push-forward uses the stored value of sigma^{n+1}
-            if constexpr (F32) sD[r * kTile + lane] = __fsub_rn((float)out[r], (float)s0r);
-            else reinterpret_cast<double*>(sD)[r * kTile + lane] = (double)out[r] - (double)s0r;
+            sD[r * kTile + lane] = __fsub_rn((float)out[r], (float)s0r);
         }
         if (active) {
 #pragma unroll
@@ -1218,7 +1137,7 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
                         __stcs(out + j * stride + (long long)cc * W * kTile, __fmaf_rn(rho, d[cc], -cj * qr[cc][j]));
                 }
             }
-        } else if constexpr (F32) {
+        } else {
             float d[CPW];
 #pragma unroll
             for (int cc = 0; cc < CPW; ++cc) d[cc] = sD[(w + cc * W) * kTile + lane];
@@ -1230,16 +1149,6 @@ __device__ __forceinline__ void compute_tile(const FwdArgs<T>& A, const StageMap
                     __stcs(out + j * stride + (long long)cc * W * kTile,
                            __fmaf_rn(rho, d[cc], -cj * qv[(j * NC + cc * W) * kTile]));
             }
-        } else {
-            double d[CPW];
-#pragma unroll
-            for (int cc = 0; cc < CPW; ++cc) d[cc] = reinterpret_cast<const double*>(sD)[(w + cc * W) * kTile + lane];
-#pragma unroll 2
-            for (int j = 0; j < m; ++j)
-#pragma unroll
-                for (int cc = 0; cc < CPW; ++cc)
-                    __stcs(out + j * stride + (long long)cc * W * kTile,
-                           (T)fma(A.mc.rho[j], d[cc], -A.mc.c[j] * (double)qv[(j * NC + cc * W) * kTile]));
         }
     }
 }
@@ -1354,10 +1263,40 @@ cudaError_t staged_smem_ready() {
     return e;
 }
 
+// The transport pre-pass of a field's two levels (ta.sig_n, ta.sig_nm1) into ta.trans.
+template <typename T, int DIM>
+cudaError_t launch_prepass(const FwdArgs<T>& ta, const LaunchCfg& cfg, cudaStream_t s) {
+    if (ta.n0 % kTX == 0 && ta.n1 % kTY == 0) {
+        // z planes per block: 16 for the staged kernel (measured at 256^3 with 3 blocks per SM:
+        // 0.39 ms against 0.45 with 8), 8 for the plain one
+        const int zs = 16, zt = 8;
+        const dim3 block(kTX, kTY);
+        if constexpr (DIM == 3) {
+            const bool staged = (long long)ta.n0 * ta.n1 < (1ll << 31) && aligned16(ta.sig_n) &&
+                                aligned16(ta.sig_nm1) && aligned16(ta.u) &&
+                                (!ta.halo_lo || (aligned16(ta.halo_lo) && aligned16(ta.halo_hi)));
+            if (staged) {
+                const cudaError_t e = staged_smem_ready<T>();
+                if (e != cudaSuccess) return e;
+                const dim3 grid(ta.n0 / kTX, ta.n1 / kTY, (ta.n2 + zs - 1) / zs);
+                transport_staged<T><<<grid, block, StagedTile<T>::kSmemBytes, s>>>(ta, cfg.stencil, zs);
+                return cudaGetLastError();
+            }
+        }
+        const dim3 grid(ta.n0 / kTX, ta.n1 / kTY, DIM == 3 ? (ta.n2 + zt - 1) / zt : 1);
+        transport_tiled<T, DIM><<<grid, block, 0, s>>>(ta, cfg.stencil, zt);
+    } else {
+        const int threads = 256;
+        long long blocks = (ta.N + threads - 1) / threads;
+        if (blocks > 152ll * 16) blocks = 152ll * 16;
+        transport_kernel<T, DIM><<<(unsigned)blocks, threads, 0, s>>>(ta, cfg.stencil);
+    }
+    return cudaGetLastError();
+}
+
 template <typename T, int DIM, bool TRANSPORT, bool COMP, bool PAPER>
 cudaError_t launch_one(const FwdArgs<T>& a, const LaunchCfg& cfg, cudaStream_t s) {
     constexpr int NC = Packed<DIM>::NC;
-    constexpr bool kQRok = sizeof(T) == 4;
     cudaError_t e;
     auto kern = fwd_kernel<T, DIM, TRANSPORT, COMP, PAPER, false>;
     const long long num_tiles = (a.N + kTile - 1) / kTile;
@@ -1379,49 +1318,20 @@ cudaError_t launch_one(const FwdArgs<T>& a, const LaunchCfg& cfg, cudaStream_t s
             ta.sig_n = a.psi_n;
             ta.sig_nm1 = a.psi_nm1;
         }
-        if (a.n0 % kTX == 0 && a.n1 % kTY == 0) {
-            // z planes per block: 16 for the staged kernel (measured at 256^3 with 3 blocks per SM:
-            // 0.39 ms against 0.45 with 8), 8 for the plain one
-            const int zs = 16, zt = 8;
-            const dim3 block(kTX, kTY);
-            bool staged = false;
-            if constexpr (DIM == 3) {
-                staged = (long long)a.n0 * a.n1 < (1ll << 31) && aligned16(ta.sig_n) && aligned16(ta.sig_nm1) &&
-                         aligned16(ta.u) &&
-                         (!ta.halo_lo || (aligned16(ta.halo_lo) && aligned16(ta.halo_hi)));
-                if (staged) {
-                    e = staged_smem_ready<T>();
-                    if (e != cudaSuccess) return e;
-                    const dim3 grid(a.n0 / kTX, a.n1 / kTY, (a.n2 + zs - 1) / zs);
-                    transport_staged<T><<<grid, block, StagedTile<T>::kSmemBytes, s>>>(ta, cfg.stencil, zs);
-                }
-            }
-            if (!staged) {
-                const dim3 grid(a.n0 / kTX, a.n1 / kTY, DIM == 3 ? (a.n2 + zt - 1) / zt : 1);
-                transport_tiled<T, DIM><<<grid, block, 0, s>>>(ta, cfg.stencil, zt);
-            }
-        } else {
-            const int threads = 256;
-            long long blocks = (a.N + threads - 1) / threads;
-            if (blocks > (long long)plan.sms * 16) blocks = (long long)plan.sms * 16;
-            transport_kernel<T, DIM><<<(unsigned)blocks, threads, 0, s>>>(ta, cfg.stencil);
-        }
-        e = cudaGetLastError();
+        e = launch_prepass<T, DIM>(ta, cfg, s);
         if (e != cudaSuccess) return e;
     }
     // one stage buffer per block: the variant that keeps Q_j in registers
     // refills the whole buffer right after the history sums
     bool qr = false;
-    if constexpr (kQRok) {
-        if (!cfg.classic && a.m <= kQR && plan.stages == 1) {
-            PersistPlan qp;
-            e = persistent_plan(reinterpret_cast<const void*>(fwd_kernel<T, DIM, TRANSPORT, COMP, PAPER, true>),
-                                32 * StepShape<DIM>::W, stage_bytes, static_bytes, 1, &qp);
-            if (e != cudaSuccess) return e;
-            if (qp.stages * qp.per_sm >= plan.stages * plan.per_sm) {
-                qr = true;
-                plan = qp;
-            }
+    if (!cfg.classic && a.m <= kQR && plan.stages == 1) {
+        PersistPlan qp;
+        e = persistent_plan(reinterpret_cast<const void*>(fwd_kernel<T, DIM, TRANSPORT, COMP, PAPER, true>),
+                            32 * StepShape<DIM>::W, stage_bytes, static_bytes, 1, &qp);
+        if (e != cudaSuccess) return e;
+        if (qp.stages * qp.per_sm >= plan.stages * plan.per_sm) {
+            qr = true;
+            plan = qp;
         }
     }
     const int stages = plan.stages;
@@ -1450,7 +1360,7 @@ cudaError_t launch_one(const FwdArgs<T>& a, const LaunchCfg& cfg, cudaStream_t s
         if (e != cudaSuccess) return e;
     }
     if (qr)
-        fwd_kernel<T, DIM, TRANSPORT, COMP, PAPER, kQRok><<<dim3((unsigned)grid), dim3(32, StepShape<DIM>::W), dyn, s>>>(
+        fwd_kernel<T, DIM, TRANSPORT, COMP, PAPER, true><<<dim3((unsigned)grid), dim3(32, StepShape<DIM>::W), dyn, s>>>(
             a, tp, 0, num_tiles, stages, vec16);
     else
         kern<<<dim3((unsigned)grid), dim3(32, StepShape<DIM>::W), dyn, s>>>(a, tp, cfg.classic ? 1 : 0, num_tiles,
@@ -1477,8 +1387,8 @@ cudaError_t dispatch(const FwdArgs<T>& a, const LaunchCfg& cfg, cudaStream_t s) 
 
 }  // namespace
 
-cudaError_t launch_forward_f64(const FwdArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s) {
-    return dispatch<double, false>(a, cfg, s);
+cudaError_t launch_prepass_f64(const FwdArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s) {
+    return cfg.dim == 2 ? launch_prepass<double, 2>(a, cfg, s) : launch_prepass<double, 3>(a, cfg, s);
 }
 
 cudaError_t launch_forward_f32(const FwdArgs<float>& a, const LaunchCfg& cfg, cudaStream_t s) {

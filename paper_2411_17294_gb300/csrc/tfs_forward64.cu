@@ -1,0 +1,544 @@
+// Forward stress step in FP64 storage: one launch advances every grid point
+// from t_n to t_{n+1} (the same step as tfs_forward.cu, which serves FP32
+// storage), all arithmetic in FP64.
+//
+// Bound.  FP64 runs at about 2 operations per clock and SM on this GPU
+// (0.5 - 0.6 T/s), so the step is bound by the number of FP64 instructions, not
+// by its bytes: 4 per (mode, component) and about 280 (3D) or 70 (2D) per point
+// for the point system.  Hence
+//   - Q'_j = x - y/4 instead of Q_j = b1 x + b2 y = -2 Q'_j, with the power of two
+//     in the constants (-2 eta_j, 2 c_j): one FMA for Q', one for the history
+//     sum, two for the push-forward, and bitwise the same values (5 before);
+//   - the transport stencil inside the step: its coefficients are formed once
+//     per point, each component then takes 3 taps per axis (the tap that the
+//     upwinding leaves out is not loaded), no separate launch, no term
+//     written and read back;
+//   - no staging of whole tiles: a warp owns one component of 32 points and
+//     loads both levels of its modes straight into registers, eight modes ahead;
+//     only Q' stays in shared memory (m nc 256 bytes, read back by the thread
+//     that wrote it).  Two to eight tiles fit an SM where the staged form held one
+//     (3D, m = 48) to four, so one tile's memory latency hides behind the others;
+//   - the point systems by FP32 LU and refinement with FP64 residuals: a thread
+//     owns one component of one point throughout, the warps of a tile factor its
+//     32 matrices in FP32 (each for itself, the FP32 pipe is idle), and each
+//     thread forms its component's residual, so a solve costs about 20 FP64
+//     operations per component and none of it waits for one warp.  FP64 Gaussian
+//     elimination with partial pivoting serves the points whose refinement does
+//     not contract, or whose numbers leave the FP32 range;
+//   - grids of few tiles split a tile's modes over several warps.
+// Measured per step (CUDA events, back to back) against the staged form this replaces: 3D 160^3,
+// m = 48: 26.7 -> 11.1 ms; 3D 192^3, m = 32 with transport: 22.9 -> 14.5 ms; 2D 1024^2, m = 32:
+// 1.18 -> 0.87 ms, with transport 1.45 -> 1.00 ms; 2D 64^2, m = 16 with transport: 27.3 -> 10.3 us.
+// The FP64 pipe is 83% (3D) and 87% (2D) busy with 927 FP64 instructions per 32-point tile at 3D,
+// m = 32.  Error against 64-bit references no larger than before (3.2e-16 against 4.8e-16 normwise
+// at 3D 160^3, 7.3e-16 against 8.9e-16 at 2D 1024^2).
+#include <cuda_runtime.h>
+
+#include "tfs_device.cuh"
+#include "tfs_internal.h"
+
+namespace tfs {
+namespace {
+
+constexpr int kT64 = 32;     // points per tile
+constexpr int kAhead = 8;    // modes whose two levels a thread loads before using them
+
+// where the transport term comes from
+enum { kNoTransport = 0, kInStep = 1, kFromPrepass = 2 };
+
+template <int DIM>
+struct Shape64 {
+    static constexpr int NC = Packed<DIM>::NC;
+    static constexpr int kSplit = 12 / NC;    // mode groups of a tile on small grids
+    static constexpr int kCoef = 3 * DIM + 1; // stencil coefficients of a point
+};
+
+template <int DIM>
+__host__ __device__ constexpr size_t smem64_bytes(int m, int groups) {
+    constexpr int NC = Packed<DIM>::NC;
+    return (size_t)kT64 * sizeof(double) *
+               ((size_t)m * NC + (size_t)groups * NC + 3 * NC + DIM * DIM + Shape64<DIM>::kCoef) +
+           (size_t)kT64 * sizeof(float) * DIM * DIM;
+}
+
+// Products of the step's scalars, formed once on the host.
+struct Step64 {
+    double scale;      // dt (the paper's variable: dt xi): what kappa* is scaled by
+    double src;        // dt G g / scale
+    double g6[3];      // dt / (6 h_a)
+    double lap[3];     // eps dt / h_a^2
+    float inv_h[3];
+    float a;
+};
+
+// Tests that keep off the FP64 pipe.
+__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool zero64(double v) {
+    return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0;
+}
+
+// v >= 0 (-0 included)
+__device__ __forceinline__ bool not_negative(double v) { return __double2hiint(v) >= 0 || zero64(v); }
+
+// Stencil coefficients of point p (times dt): per axis the taps at -1, +1 and at
+// the far upwind point, then the centre, into cf[k * 32].  Returns sum_a |u_a| / h_a.
+template <int DIM>
+__device__ __forceinline__ float stencil_coefs(const FwdArgs<double>& A, const Step64& B, int stencil, const double u[DIM],
+                                               double* cf) {
+    double c0 = 0.0;
+    float cr = 0.0f;
+#pragma unroll
+    for (int ax = 0; ax < DIM; ++ax) {
+        const double g = u[ax] * B.g6[ax];
+        double lo, hi, far;
+        if (stencil == 1) {
+            lo = -3.0 * g;
+            hi = 3.0 * g;
+            far = 0.0;
+        } else {
+            const bool pos = not_negative(u[ax]);
+            lo = g * (pos ? -6.0 : -2.0);
+            hi = g * (pos ? 2.0 : 6.0);
+            far = pos ? g : -g;
+            c0 = fma(g, pos ? 3.0 : -3.0, c0);
+        }
+        if (A.eps != 0.0) {
+            lo -= B.lap[ax];
+            hi -= B.lap[ax];
+            c0 = fma(2.0, B.lap[ax], c0);
+        }
+        cf[(3 * ax + 0) * kT64] = lo;
+        cf[(3 * ax + 1) * kT64] = hi;
+        cf[(3 * ax + 2) * kT64] = far;
+        cr += fabsf((float)u[ax]) * B.inv_h[ax];
+    }
+    cf[3 * DIM * kT64] = c0;
+    return cr;
+}
+
+// The transport term of component c at point p from the coefficients in cf.
+template <int DIM>
+__device__ __forceinline__ double stencil_term(const FwdArgs<double>& A, int stencil, int c, long long p,
+                                               const double* cf) {
+    constexpr int NC = Packed<DIM>::NC;
+    const unsigned pu = (unsigned)p;
+    const int nn[3] = {A.n0, A.n1, A.n2};
+    const unsigned r1 = pu / (unsigned)A.n0;
+    const int co[3] = {(int)(pu % (unsigned)A.n0), (int)(DIM == 3 ? r1 % (unsigned)A.n1 : r1),
+                       (int)(DIM == 3 ? r1 / (unsigned)A.n1 : 0)};
+    const long long stride[3] = {1, A.n0, (long long)A.n0 * A.n1};
+    const double* sn = A.sig_n + (long long)c * A.N;
+    const double* sm = A.sig_nm1 + (long long)c * A.N;
+    // E = 2 sigma^n - sigma^{n-1} at offset off along axis ax: periodic wrap, or on a slab
+    // the slowest axis beyond the grid from the halo planes
+    auto at = [&](int ax, int off) -> double {
+        int v = co[ax] + off;
+        if ((v < 0 || v >= nn[ax]) && ax == DIM - 1 && A.halo_lo) {
+            const long long pl = stride[DIM - 1];
+            const double* hb = v < 0 ? A.halo_lo : A.halo_hi;
+            const int k = v < 0 ? v + A.halo_r : v - nn[ax];
+            const long long q = ((long long)c * A.halo_r + k) * pl + (p - (long long)co[ax] * pl);
+            return fma(2.0, __ldg(hb + q), -__ldg(hb + (long long)NC * A.halo_r * pl + q));
+        }
+        if (v < 0) v += nn[ax];
+        if (v < 0) v += nn[ax];
+        if (v >= nn[ax]) v -= nn[ax];
+        if (v >= nn[ax]) v -= nn[ax];
+        const long long q = p + (long long)(v - co[ax]) * stride[ax];
+        return fma(2.0, __ldg(sn + q), -__ldg(sm + q));
+    };
+    double acc = cf[3 * DIM * kT64] * fma(2.0, __ldg(sn + p), -__ldg(sm + p));
+#pragma unroll
+    for (int ax = 0; ax < DIM; ++ax) {
+        const double lo = at(ax, -1), hi = at(ax, 1);
+        acc = fma(cf[(3 * ax + 0) * kT64], lo, acc);
+        acc = fma(cf[(3 * ax + 1) * kT64], hi, acc);
+        if (stencil == 0) {
+            // the sign of the coefficient is that of u (far = g or -g: u >= 0 takes the tap at -2)
+            const double fc = cf[(3 * ax + 2) * kT64];
+            const double ua = __ldg(A.u + (long long)ax * A.N + p);
+            acc = fma(fc, at(ax, not_negative(ua) ? -2 : 2), acc);
+        }
+    }
+    return acc;
+}
+
+// ---- FP32 images of FP64 numbers by integer operations (a conversion costs what
+// an FP64 operation does).  A vector is scaled by the power of two that brings
+// its largest component to [1, 2); smaller components lose the bits below that
+// of the float format, which the refinement recovers.
+__device__ __forceinline__ int biased_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+__device__ __forceinline__ float scaled_float(double v, int emax) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const int be = (hi >> 20) & 0x7ff, e = be - emax + 127;
+    const unsigned bits = ((unsigned)hi & 0x80000000u) | ((unsigned)e << 23) | (((unsigned)hi & 0xfffffu) << 3) |
+                          ((unsigned)lo >> 29);
+    return be > 0 && e > 0 ? __uint_as_float(bits) : 0.0f;
+}
+
+// f 2^(emax - 1023), exactly, for a finite f whose scaled exponent is in range (0 below it).
+__device__ __forceinline__ double unscaled_double(float f, int emax) {
+    const unsigned b = __float_as_uint(f);
+    const int e = (int)((b >> 23) & 0xffu) - 127 + emax;
+    const int hi = (int)((b & 0x80000000u) | ((unsigned)e << 20) | ((b & 0x7fffffu) >> 3));
+    return ((b >> 23) & 0xffu) != 0u && e > 0 ? __hiloint2double(hi, (int)(b << 29)) : 0.0;
+}
+
+// Barrier of the first N threads of a block.
+template <int N>
+__device__ __forceinline__ void named_sync() {
+    asm volatile("bar.sync 1, %0;\n" ::"n"(N) : "memory");
+}
+
+// Packed component of the symmetric entry (a, b).
+template <int DIM>
+struct PackedIndex {
+    __host__ __device__ static constexpr int at(int a, int b) {
+        return a == b ? (DIM == 2 ? 2 * a : a) : (DIM == 2 ? 1 : 6 - a - b);
+    }
+};
+
+// The point system by FP64 Gaussian elimination (K scaled as in the kernel):
+// component c of M^-1 R.  Returns false when a pivot vanishes.
+template <int DIM>
+__device__ __noinline__ bool solve_by_elimination(const double* sK, const double* sR, double a, int c, double* out) {
+    constexpr int NC = Packed<DIM>::NC;
+    double K[3][3], x[NC], M[NC][NC];
+#pragma unroll
+    for (int i = 0; i < DIM; ++i)
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) K[i][j] = sK[(i * DIM + j) * kT64];
+#pragma unroll
+    for (int r = 0; r < NC; ++r) x[r] = sR[r * kT64];
+    assemble_M<DIM>(K, a, 1.0, M);
+    const bool ok = gauss_pp<NC>(M, x, 1e-300);
+    *out = x[0];
+#pragma unroll
+    for (int r = 1; r < NC; ++r)
+        if (c == r) *out = x[r];
+    return ok;
+}
+
+// One tile of 32 points per block; warp (c, g) takes component c and the modes
+// j = g mod G, and with g = 0 the component's part of the point systems.
+template <int DIM, int TR, bool PAPER, int G>
+__global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 2 ? 8 : 3))
+    fwd64_kernel(const FwdArgs<double> A, const Step64 B, const int classic, const int stencil) {
+    constexpr int NC = Packed<DIM>::NC;
+    constexpr int DD = DIM * DIM;
+    extern __shared__ __align__(16) double sm64[];
+    const int lane = threadIdx.x;
+    const int w = threadIdx.y;
+    const int c = w % NC, grp = w / NC;
+    const int m = classic ? 0 : A.m;
+    double* sQ = sm64;                          // Q'_j [m][NC][32]
+    double* sH = sQ + (size_t)m * NC * kT64;    // partial history sums [G][NC][32]
+    double* sR = sH + G * NC * kT64;            // right-hand side, then two buffers of residuals [3][NC][32]
+    double* sK = sR + 3 * NC * kT64;            // dt kappa* (the paper's variable: dt xi kappa*) [DD][32]
+    double* sC = sK + DD * kT64;                // stencil coefficients
+    float* sKf = reinterpret_cast<float*>(sC + Shape64<DIM>::kCoef * kT64);   // sK in FP32
+    const long long t0 = (long long)blockIdx.x * kT64;
+    const long long p = t0 + lane;
+    const bool active = p < A.N;
+    const long long pc = active ? p : A.N - 1;  // a point to read where the tile ends past the grid
+    const bool has_s0 = A.sigma0 != nullptr;
+
+    // ---- velocity gradient entries and stencil coefficients, spread over the warps
+    for (int k = w; k < DD; k += NC * G) {
+        const long long q = (long long)k * A.N + pc;
+        const double v = B.scale * fma(2.0, A.kap_n[q], -A.kap_nm1[q]);
+        sK[k * kT64 + lane] = v;
+        sKf[k * kT64 + lane] = (float)v;
+    }
+    if (TR == kInStep && w == NC * G - 1) {
+        double u[DIM];
+#pragma unroll
+        for (int ax = 0; ax < DIM; ++ax) u[ax] = __ldg(A.u + (long long)ax * A.N + pc);
+        const float cr = stencil_coefs<DIM>(A, B, stencil, u, sC + lane);
+        const float ccoef = (float)A.courant_coef;
+        const bool over = active && ccoef > 0.0f && ccoef * cr > (float)A.courant_limit;
+        if (__any_sync(0xffffffffu, over) && lane == 0) atomicOr(A.flags, 4u);
+    }
+
+    // ---- history sum over this warp's modes (constants: -2 eta_j in mc.eta): one partial
+    //      sum per residue of j mod kSplit, added in the order of the residues, whether
+    //      one warp holds them all or each has its own (a slab of a domain may be split
+    //      where the domain is not, and gives the same bits)
+    constexpr int kSums = Shape64<DIM>::kSplit / G;
+    double part[kSums];
+#pragma unroll
+    for (int k = 0; k < kSums; ++k) part[k] = 0.0;
+    if (classic) {
+        if (grp == 0) {
+            const long long q = (long long)c * A.N + pc;
+            part[0] = kB1 * A.sig_n[q] + kB2 * A.sig_nm1[q] + (has_s0 ? kB0 * A.sigma0[q] : 0.0);
+        }
+    } else {
+        constexpr long long row = (long long)NC * kT64;
+        const long long base = mode_index(t0, c, m * NC) + lane;
+        const double* xs = A.modes_n + base;
+        const double* ys = A.modes_nm1 + base;
+        double* q = sQ + c * kT64 + lane;
+#pragma unroll 1
+        for (int jb = grp; jb < m; jb += G * kAhead) {
+            double x[kAhead], y[kAhead];
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) {
+                const int j = jb + k * G;
+                if (j < m) {
+                    x[k] = __ldcs(xs + j * row);
+                    y[k] = __ldcs(ys + j * row);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) {
+                const int j = jb + k * G;
+                if (j < m) {
+                    const double qp = fma(-0.25, y[k], x[k]);
+                    part[k % kSums] = fma(A.mc.eta[j], qp, part[k % kSums]);
+                    q[j * row] = qp;
+                }
+            }
+        }
+    }
+    double H = part[0];
+#pragma unroll
+    for (int k = 1; k < kSums; ++k) H += part[k];
+    if (G > 1 || PAPER) sH[(grp * NC + c) * kT64 + lane] = H;
+    __syncthreads();
+
+    // ---- right-hand side of this thread's component
+    double x = 0.0, r = 0.0, s0 = 0.0;
+    const int ci = Packed<DIM>::I(c), cj = Packed<DIM>::J(c);
+    if (grp == 0) {
+#pragma unroll
+        for (int g = 1; g < G; ++g) H += sH[(g * NC + c) * kT64 + lane];
+        const long long q = (long long)c * A.N + pc;
+        const double ks = sK[(ci * DIM + cj) * kT64 + lane] + sK[(cj * DIM + ci) * kT64 + lane];
+        if constexpr (PAPER) {
+            // -b1 Phi^n - b2 Phi^{n-1} + dt (L(kappa*) h - h/Wi) + dt G (kappa* + kappa*^T) Psi0 [- A]
+            // against (b0 + dt xi/Wi) Phi - dt xi L(kappa*) Phi; h_ab of the other components
+            // from shared memory (their partial sums, added in the same order)
+            auto hat = [&](int a, int b) {
+                const int k = PackedIndex<DIM>::at(a, b);
+                double v = sH[k * kT64 + lane];
+#pragma unroll
+                for (int g = 1; g < G; ++g) v += sH[(g * NC + k) * kT64 + lane];
+                return v;
+            };
+            double lh = 0.0;
+#pragma unroll
+            for (int l = 0; l < DIM; ++l)
+                lh = fma(sK[(ci * DIM + l) * kT64 + lane], hat(l, cj),
+                         fma(hat(ci, l), sK[(cj * DIM + l) * kT64 + lane], lh));
+            // (sK carries dt xi; A.eta holds 1/xi in this variable)
+            r = fma(2.0, A.sig_n[q], -0.5 * A.sig_nm1[q]) - A.dt * A.inv_wi * H + fma(B.src, ks, A.eta * lh);
+            if (TR == kFromPrepass) r -= A.trans[q];
+        } else {
+            s0 = has_s0 ? A.sigma0[q] : 0.0;
+            r = fma(B.src, ks, fma(A.eta, s0, -H));
+            if (TR == kInStep) r -= stencil_term<DIM>(A, stencil, c, pc, sC + lane);
+        }
+        sR[c * kT64 + lane] = r;
+    }
+    __syncthreads();
+    if (grp == 0) {
+        // ---- FP32 factors of the 32 matrices, one each per lane, in every warp
+        LU32<NC> F;
+        static_for<0, NC>([&](auto rr) {
+            constexpr int ro = decltype(rr)::value;
+            static_for<0, NC>([&](auto kk) {
+                constexpr int k = decltype(kk)::value;
+                constexpr int i1 = Packed<DIM>::I(ro), j1 = Packed<DIM>::J(ro);
+                constexpr int i = Packed<DIM>::I(k), j = Packed<DIM>::J(k);
+                const float* kf = sKf + lane;
+                float v = ro == k ? B.a : 0.0f;
+                if (j1 == j) v -= kf[(i1 * DIM + i) * kT64];
+                if (i != j && j1 == i) v -= kf[(i1 * DIM + j) * kT64];
+                if (i1 == i) v -= kf[(j1 * DIM + j) * kT64];
+                if (i != j && i1 == j) v -= kf[(j1 * DIM + i) * kT64];
+                F.a[ro][k] = v;
+            });
+        });
+        bool good = row_dominant<NC>(F) ? lu32_factor_nopivot<NC>(F, 1e-30f) : lu32_factor<NC>(F, 1e-30f);
+        // ---- x = y0 + y1 + y2 ...: each y the FP32 solution for the residual so far.  With
+        //      contraction q per pass the error after y2 is |y2| q: q < 2^-18 leaves it below
+        //      the last bit, and then |y2| is below 2^-36 |x|; otherwise further passes
+        int e0 = 0;
+        constexpr int kMaxPass = 8;
+        bool done = false;
+        for (int pass = 0; pass < kMaxPass; ++pass) {
+            const double* rb = pass == 0 ? sR : sR + (1 + (pass & 1)) * NC * kT64;
+            double rv[NC];
+            int emax = 0;
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                rv[k] = rb[k * kT64 + lane];
+                emax = max(emax, biased_exp(rv[k]));
+            }
+            // a residual of zeros (or below the range of a scaled float) is solved
+            bool zero = true;
+            float y[NC];
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                zero = zero && zero64(rv[k]);
+                y[k] = scaled_float(rv[k], emax);
+            }
+            if (pass == 0) good = good && emax < 0x7ff && (emax > 200 || zero);
+            lu32_solve<NC>(F, y);
+            unsigned ymax = 0u;
+#pragma unroll
+            for (int k = 0; k < NC; ++k) ymax = max(ymax, __float_as_uint(y[k]) & 0x7fffffffu);
+            const int ey = (int)(ymax >> 23) + emax;       // exponent of the correction (biased by 127 + 1023)
+            if (pass == 0) {
+                good = good && ymax < 0x7f800000u && ey - 127 < 0x7ff;
+                e0 = ey;
+            }
+            const bool small = ymax == 0u || ey <= e0 - 36;
+            static_for<0, NC>([&](auto kk) {
+                constexpr int k = decltype(kk)::value;
+                // a point's passes are its own, whatever the other points of its tile still need
+                if (c == k && !done) x += unscaled_double(y[k], emax);
+            });
+            done = done || zero || (pass >= 2 && small);
+            if (__all_sync(0xffffffffu, done || !good)) break;
+            static_for<0, NC>([&](auto kk) {
+                constexpr int k = decltype(kk)::value;
+                if (c == k) {
+                    constexpr int i = Packed<DIM>::I(k), j = Packed<DIM>::J(k);
+                    r = fma(-A.a, unscaled_double(y[k], emax), r);
+                    static_for<0, DIM>([&](auto ll) {
+                        constexpr int l = decltype(ll)::value;
+                        constexpr int lj = PackedIndex<DIM>::at(l, j), li = PackedIndex<DIM>::at(l, i);
+                        r = fma(sK[(i * DIM + l) * kT64 + lane], unscaled_double(y[lj], emax), r);
+                        r = fma(sK[(j * DIM + l) * kT64 + lane], unscaled_double(y[li], emax), r);
+                    });
+                }
+            });
+            sR[(1 + ((pass + 1) & 1)) * NC * kT64 + c * kT64 + lane] = r;
+            named_sync<NC * 32>();
+        }
+        unsigned fl = 0u;
+        if (!good || !done) {
+            if (!solve_by_elimination<DIM>(sK + lane, sR + lane, A.a, c, &x) && active) fl |= 2u;
+        }
+        const long long q = (long long)c * A.N + p;
+        bool finite = finite64(x);
+        if (active) {
+            A.sig_np1[q] = x;
+            if constexpr (PAPER) {
+                const double psi = fma(A.xi, x, H);
+                finite = finite && finite64(psi);
+                A.psi[q] = psi;
+                if (A.sig_copy) A.sig_copy[q] = psi;
+            } else {
+                if (A.sig_copy) A.sig_copy[q] = x;
+            }
+            if (!finite) fl |= 1u;
+            if (fl) atomicOr(A.flags, fl);
+        }
+        x -= s0;
+        if (G > 1) sH[c * kT64 + lane] = x;
+    }
+    if (G > 1) {
+        __syncthreads();
+        x = sH[c * kT64 + lane];
+    }
+
+    // ---- push-forward over the oldest level (constants: 2 c_j in mc.c)
+    if (!classic && active) {
+        constexpr long long row = (long long)NC * kT64;
+        const double* q = sQ + c * kT64 + lane;
+        double* out = A.modes_nm1 + mode_index(p, c, m * NC);
+#pragma unroll 4
+        for (int j = grp; j < m; j += G) __stcs(out + j * row, fma(A.mc.rho[j], x, A.mc.c[j] * q[j * row]));
+    }
+}
+
+// Raises a kernel's dynamic shared-memory limit once per device.
+template <int DIM, int TR, bool PAPER, int G>
+cudaError_t smem_ready() {
+    static bool done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
+    e = cudaFuncSetAttribute(fwd64_kernel<DIM, TR, PAPER, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem64_bytes<DIM>(kMaxModes, G));
+    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
+    return e;
+}
+
+template <int DIM, int TR, bool PAPER, int G>
+cudaError_t launch64(const FwdArgs<double>& a, const LaunchCfg& cfg, long long tiles, cudaStream_t s) {
+    cudaError_t e = smem_ready<DIM, TR, PAPER, G>();
+    if (e != cudaSuccess) return e;
+    const size_t dyn = smem64_bytes<DIM>(cfg.classic ? 0 : a.m, G);
+    Step64 b;
+    b.scale = PAPER ? a.dt * a.xi : a.dt;
+    b.src = PAPER ? a.G * a.g / a.xi : a.G * a.g;
+    for (int i = 0; i < 3; ++i) {
+        b.g6[i] = a.dt * a.inv_h[i] / 6.0;
+        b.lap[i] = a.eps * a.dt * a.inv_h[i] * a.inv_h[i];
+        b.inv_h[i] = (float)a.inv_h[i];
+    }
+    b.a = (float)a.a;
+    fwd64_kernel<DIM, TR, PAPER, G><<<(unsigned)tiles, dim3(kT64, Packed<DIM>::NC * G), dyn, s>>>(
+        a, b, cfg.classic ? 1 : 0, cfg.stencil);
+    return cudaGetLastError();
+}
+
+// Tiles up to which a tile's modes are split over several warps: one block per SM.  Measured, split
+// against not: 128 tiles (2D 64^2, m = 16, with transport) 10.3 us against 12.2; beyond it 288 tiles
+// 14.2 against 12.4, 480 (m = 24) 20.5 against 16.4, 512 (m = 32) 26.6 against 23.1; 3D, 183 tiles
+// (m = 24) 24.2 against 18.5.
+constexpr long long kSplitTiles = 152;
+
+template <int DIM, int TR, bool PAPER>
+cudaError_t launch_split(const FwdArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s) {
+    const long long tiles = (a.N + kT64 - 1) / kT64;
+    if (tiles <= kSplitTiles) return launch64<DIM, TR, PAPER, Shape64<DIM>::kSplit>(a, cfg, tiles, s);
+    return launch64<DIM, TR, PAPER, 1>(a, cfg, tiles, s);
+}
+
+template <int DIM>
+cudaError_t launch_dim(const FwdArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s) {
+    if (cfg.paper) {
+        if (cfg.transport) return launch_split<DIM, kFromPrepass, true>(a, cfg, s);
+        return launch_split<DIM, kNoTransport, true>(a, cfg, s);
+    }
+    if (cfg.transport) return launch_split<DIM, kInStep, false>(a, cfg, s);
+    return launch_split<DIM, kNoTransport, false>(a, cfg, s);
+}
+
+}  // namespace
+
+cudaError_t launch_forward_f64(const FwdArgs<double>& args, const LaunchCfg& cfg, cudaStream_t s) {
+    if (cfg.paper && (cfg.classic || !args.psi)) return cudaErrorInvalidValue;
+    if (cfg.paper && cfg.transport) {
+        // Psi^{n+1} is written over Psi^{n-1}, which its neighbours' stencils
+        // still need: this variable keeps the pre-pass
+        if (!args.psi_n || !args.psi_nm1 || !args.trans) return cudaErrorInvalidValue;
+        FwdArgs<double> ta = args;
+        ta.sig_n = args.psi_n;
+        ta.sig_nm1 = args.psi_nm1;
+        const cudaError_t e = launch_prepass_f64(ta, cfg, s);
+        if (e != cudaSuccess) return e;
+    }
+    FwdArgs<double> a = args;
+    if (cfg.paper) a.eta = 1.0 / a.xi;
+    for (int j = 0; j < a.m; ++j) {   // Q = -2 Q'
+        a.mc.c[j] *= 2.0;
+        a.mc.eta[j] *= -2.0;
+    }
+    if (cfg.ev_before) {
+        const cudaError_t e = cudaEventRecord(cfg.ev_before, s);
+        if (e != cudaSuccess) return e;
+    }
+    cudaError_t e = cfg.dim == 2 ? launch_dim<2>(a, cfg, s) : launch_dim<3>(a, cfg, s);
+    if (e == cudaSuccess && cfg.ev_after) e = cudaEventRecord(cfg.ev_after, s);
+    return e;
+}
+
+}  // namespace tfs

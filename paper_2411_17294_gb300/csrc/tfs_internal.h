@@ -244,9 +244,11 @@ struct LaunchCfg {
     cudaEvent_t ev_after = nullptr;    // (not around the transport pre-pass), if set
 };
 
-// forward launchers (tfs_forward.cu)
+// forward launchers: FP64 storage (tfs_forward64.cu), FP32 storage and the FP64
+// transport pre-pass of the paper's variable (tfs_forward.cu)
 cudaError_t launch_forward_f64(const FwdArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s);
 cudaError_t launch_forward_f32(const FwdArgs<float>& a, const LaunchCfg& cfg, cudaStream_t s);
+cudaError_t launch_prepass_f64(const FwdArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s);
 
 // Arguments of one adjoint step launch (see tfs_adjoint.cu).
 template <typename T>

@@ -230,6 +230,17 @@ int tfs_step(tfs_handle h, const void* grad_u_n, const void* grad_u_nm1, const v
    `stream`; TFS_ERR_STATE before tfs_set_state. */
 int tfs_get_stress(tfs_handle h, void* out, void* stream);
 
+/* `steps` steps with a frozen velocity gradient (kappa^n = kappa^{n-1} =
+   grad_u; u when transport is on), with the results of that many tfs_step
+   calls: trajectory [steps][nc][N] (device, element type of the handle, 16-byte
+   aligned) receives the stress after each step (Psi with TFS_FORM_PAPER), and
+   the state is that after the last.  The FP32 stress form with alpha < 1, BDF2
+   start and transport 0 keeps its modes in registers over the steps (bitwise
+   the same stresses).  Enqueues on `stream` (implicit transport synchronises);
+   errors as tfs_step, TFS_ERR_ARG for steps < 1 or a NULL or misaligned
+   trajectory. */
+int tfs_run(tfs_handle h, int steps, const void* grad_u, const void* u, void* trajectory, void* stream);
+
 /* Slab decomposition (for running one periodic domain on several GPUs).  The
    paper's runtime partitions its meshes over MPI ranks (Section 5, the
    experimental setup); this is the library's counterpart for the periodic
@@ -322,6 +333,15 @@ int tfs_bind_adjoint_workspace(tfs_handle h, void* dev_ptr, size_t bytes);
 int tfs_backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* checkpoints, int K,
                  int steps, const void* grad_u, const void* u, double* dJ_dsigma0,
                  double* dJ_dgrad_u, double* dJ_dWi, double* dJ_dbeta, void* stream);
+
+/* The same derivatives from the trajectory of all `steps` steps that tfs_run wrote from
+   the state set by tfs_set_state, so that nothing is recomputed (the handle's
+   forward state is left alone).  The adjoint workspace may be bound for one
+   segment step.  TFS_ERR_ARG with implicit transport or the SDIRK2 start, whose reverse steps
+   need the state itself (tfs_backward). */
+int tfs_backward_run(tfs_handle h, const void* dJ_dsigma_T, const void* trajectory, int steps, const void* grad_u,
+                     const void* u, double* dJ_dsigma0, double* dJ_dgrad_u, double* dJ_dWi, double* dJ_dbeta,
+                     void* stream);
 
 /* Read (and keep) the latched device flags; synchronises the last stream
    the handle used.  Returns TFS_OK or TFS_ERR_CUDA. */

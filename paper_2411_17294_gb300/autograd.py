@@ -2,11 +2,13 @@
 
 ``fractional_stress(sigma0, grad_u, Wi, beta, ...)`` advances the stress
 ``steps`` steps with a frozen velocity gradient and returns sigma(T).  Its
-backward is the library's hand-written adjoint (tfs_backward): the forward
-keeps a full-state checkpoint every K steps (the mode history is m times the
-stress and is not stored); the backward recomputes each K-step segment from its
-checkpoint and sweeps it in reverse.  Gradients flow to sigma0, grad_u, Wi and
-beta.
+backward is the library's hand-written adjoint.  The reverse sweep needs the
+stress after each step, not the modes.  Where storing that costs no more memory
+than full-state checkpoints every K steps would (a checkpoint holds both mode
+levels, 2 m + 3 stress fields), the forward keeps the stresses of all steps and the
+backward recomputes nothing (tfs_run, tfs_backward_run); longer runs, implicit
+transport and the SDIRK2 start keep the checkpoints, and the backward recomputes
+each K-step segment (tfs_backward).  Gradients flow to sigma0, grad_u, Wi and beta.
 """
 from __future__ import annotations
 
@@ -30,8 +32,13 @@ class TFSFunction(torch.autograd.Function):
         kt = grad_u.detach().to(s.dtype).reshape(dim * dim, -1).contiguous()
         ut = u.detach().to(s.dtype).reshape(dim, -1).contiguous() if transport else None
         s.set_state(sigma0.detach())
-        ckpts = []
-        for k in range(steps):
+        segments = -(-steps // K)
+        whole = (0 < steps <= segments * (2 * s.m + 3) and transport != "implicit"
+                 and cfg.get("start", "bdf2") == "bdf2")
+        ckpts, traj = [], None
+        if whole:
+            traj = s.run(steps, kt, ut)
+        for k in range(0 if whole else steps):
             if k % K == 0:
                 buf = s.new_checkpoint()
                 s.save(buf)
@@ -39,7 +46,7 @@ class TFSFunction(torch.autograd.Function):
             s.step(kt, kt, ut)
         out = s.stress().to(sigma0.dtype).reshape(sigma0.shape)
         ctx.solver = s
-        ctx.ckpts = ckpts
+        ctx.ckpts, ctx.traj = ckpts, traj
         ctx.kt, ctx.ut = kt, ut
         ctx.meta = (steps, K, sigma0.dtype, sigma0.shape, grad_u.dtype, grad_u.shape, Wi, beta)
         return out
@@ -48,10 +55,14 @@ class TFSFunction(torch.autograd.Function):
     def backward(ctx, g_out):
         steps, K, s_dtype, s_shape, k_dtype, k_shape, Wi, beta = ctx.meta
         s = ctx.solver
-        g_s0, g_k, gWi, gb = s.backward(g_out.detach().reshape(s.nc, -1), ctx.ckpts, K, steps, ctx.kt, ctx.ut)
+        dJ = g_out.detach().reshape(s.nc, -1)
+        if ctx.traj is not None:
+            g_s0, g_k, gWi, gb = s.backward_run(dJ, ctx.traj, ctx.kt, ctx.ut)
+        else:
+            g_s0, g_k, gWi, gb = s.backward(dJ, ctx.ckpts, K, steps, ctx.kt, ctx.ut)
         s.close()
         ctx.solver = None
-        ctx.ckpts = None
+        ctx.ckpts = ctx.traj = None
         dWi = torch.tensor(gWi, dtype=Wi.dtype, device=Wi.device) if isinstance(Wi, torch.Tensor) else None
         db = torch.tensor(gb, dtype=beta.dtype, device=beta.device) if isinstance(beta, torch.Tensor) else None
         return (g_s0.to(s_dtype).reshape(s_shape), g_k.to(k_dtype).reshape(k_shape), dWi, db, None, None)

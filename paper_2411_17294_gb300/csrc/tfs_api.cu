@@ -13,6 +13,7 @@
 
 #include "../../include/tfs.h"
 #include "tfs_internal.h"
+#include "tfs_resident.h"
 #include "tfs_adjoint_paper.h"
 #include "tfs_adjoint_implicit.h"
 
@@ -753,13 +754,20 @@ int do_first_step_sdirk2(tfs_ctx* h, const void* kn, const void* u, void* sig_co
     return TFS_OK;
 }
 
-int do_step(tfs_ctx* h, const void* kn, const void* knm1, const void* u, void* sig_copy, cudaStream_t s) {
+// What refuses a step before it starts.
+int step_refused(tfs_ctx* h, const void* kn, const void* u) {
     if (!h->ws) return TFS_ERR_NOWORKSPACE;
     if (!h->state_set) return TFS_ERR_STATE;
     if (!h->classic() && !h->soe_set) return TFS_ERR_NOSOE;
     if (!kn) return TFS_ERR_ARG;
     if (h->transport && !u) return TFS_ERR_ARG;
     if (limits_violated(h)) return TFS_ERR_UNSTABLE;
+    return TFS_OK;
+}
+
+int do_step(tfs_ctx* h, const void* kn, const void* knm1, const void* u, void* sig_copy, cudaStream_t s) {
+    const int refused = step_refused(h, kn, u);
+    if (refused != TFS_OK) return refused;
     if (!knm1) knm1 = kn;
     if (h->start == TFS_START_SDIRK2 && h->step == 0) return do_first_step_sdirk2(h, kn, u, sig_copy, s);
     if (h->implicit_transport()) return do_step_implicit(h, kn, knm1, u, sig_copy, s);
@@ -829,6 +837,93 @@ int do_step(tfs_ctx* h, const void* kn, const void* knm1, const void* u, void* s
     h->step += 1;
     h->last_stream = s;
     return TFS_OK;
+}
+
+// ---------------------------- many steps in one launch (tfs_resident.cu)
+// FP32 storage, the stress form, alpha < 1, BDF2 start, pointwise law.
+bool resident_path(const tfs_ctx* h) {
+    return !h->is_double() && !h->classic() && !h->paper() && h->transport == 0 && h->start == TFS_START_BDF2;
+}
+
+// `steps` steps with a frozen velocity gradient; sigma^{n+1} of step k goes to
+// rows + k stride (bytes).
+int run_resident(tfs_ctx* h, int steps, const void* grad_u, char* rows, size_t stride, cudaStream_t s) {
+    ResidentRun a{};
+    a.kap = (const float*)grad_u;
+    a.sigma0 = h->sigma0_zero ? nullptr : (const float*)h->sigma0;
+    a.modes_n = (float*)h->modes[h->cur_mode];
+    a.modes_nm1 = (float*)h->modes[1 - h->cur_mode];
+    a.stride = (long long)(stride / sizeof(float));
+    a.flags = h->flags;
+    a.N = h->N;
+    a.m = h->m;
+    a.mc = h->mcf;
+    a.eta = split_f2(h->eta);
+    a.a = split_f2(h->eta + h->dt / h->Wi);
+    a.dt = split_f2(h->dt);
+    const double G = (1.0 - h->beta) / (h->Wi * h->Re);
+    cudaError_t e = cudaSuccess;
+    for (int k0 = 0; k0 < steps && e == cudaSuccess; k0 += kRunSteps) {
+        a.steps = steps - k0 < kRunSteps ? steps - k0 : kRunSteps;
+        a.rows = (float*)(rows + (size_t)k0 * stride);
+        for (int k = 0; k < a.steps; ++k) a.src[k] = split_f2(h->dt * G * g_alpha(h, h->step + k0 + k));
+        e = launch_resident_run(a, h->dim, h->precision == TFS_FP32, s);
+    }
+    // the stress ring as after the last step
+    const int older = h->cur_sig, newest = h->prev_sig;
+    if (steps >= 2 && e == cudaSuccess)
+        e = cudaMemcpyAsync(h->sig[older], rows + (size_t)(steps - 2) * stride, h->field_bytes(),
+                            cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h->sig[newest], rows + (size_t)(steps - 1) * stride, h->field_bytes(),
+                            cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) return TFS_ERR_CUDA;
+    h->cur_sig = newest;
+    h->prev_sig = older;
+    h->step += steps;
+    h->last_stream = s;
+    return TFS_OK;
+}
+
+// Reverse of steps [start, end) from their stresses; dJ: the adjoint of the final
+// stress when end is the last step, else nullptr.
+cudaError_t back_resident(const tfs_ctx* h, int start, int end, const void* grad_u, const char* rows, size_t stride,
+                          const void* dJ, char* ell_prev, char* ell_prev2, double* g_sigma0, double* g_kap,
+                          double* partials, cudaStream_t s) {
+    ResidentBack a{};
+    a.kap = (const float*)grad_u;
+    a.stride = (long long)(stride / sizeof(float));
+    a.ell_prev = (float*)ell_prev;
+    a.ell_prev2 = (float*)ell_prev2;
+    a.g_sigma0 = g_sigma0;
+    a.g_kap = g_kap;
+    a.partials = partials;
+    a.flags = h->flags;
+    a.N = h->N;
+    a.m = h->m;
+    a.mc = h->mcf;
+    a.eta = split_f2(h->eta);
+    a.a = (float)(h->eta + h->dt / h->Wi);
+    a.dt = (float)h->dt;
+    const double G = (1.0 - h->beta) / (h->Wi * h->Re);
+    a.dt_wi2 = h->dt / (h->Wi * h->Wi);
+    a.g_wi = G / h->Wi;
+    a.inv_wire = 1.0 / (h->Wi * h->Re);
+    cudaError_t e = cudaSuccess;
+    for (int top = end; top > start && e == cudaSuccess;) {
+        a.steps = top - start < kRunSteps ? top - start : kRunSteps;
+        const int first = top - a.steps;
+        a.rows = (const float*)(rows + (size_t)(first - start) * stride);
+        a.dJ = top == end ? (const float*)dJ : nullptr;
+        for (int k = 0; k < a.steps; ++k) {
+            const double g = g_alpha(h, top - 1 - k);
+            a.src[k] = (float)(h->dt * G * g);
+            a.dtg[k] = split_f2(h->dt * g);
+        }
+        e = launch_resident_back(a, h->dim, s);
+        top = first;
+    }
+    return e;
 }
 
 bool valid_handle(tfs_handle h) { return h != nullptr; }
@@ -1042,6 +1137,21 @@ int tfs_set_state(tfs_handle h, const void* sigma0, void* stream) {
 int tfs_step(tfs_handle h, const void* grad_u_n, const void* grad_u_nm1, const void* u, void* stream) {
     if (!valid_handle(h)) return TFS_ERR_ARG;
     return do_step(h, grad_u_n, grad_u_nm1, u, nullptr, (cudaStream_t)stream);
+}
+
+int tfs_run(tfs_handle h, int steps, const void* grad_u, const void* u, void* trajectory, void* stream) {
+    if (!valid_handle(h) || steps < 1 || !trajectory || ((uintptr_t)trajectory) % 16) return TFS_ERR_ARG;
+    char* rows = (char*)trajectory;
+    const size_t stride = h->field_bytes();
+    if (resident_path(h)) {
+        const int rc = step_refused(h, grad_u, u);
+        return rc != TFS_OK ? rc : run_resident(h, steps, grad_u, rows, stride, (cudaStream_t)stream);
+    }
+    for (int k = 0; k < steps; ++k) {
+        const int rc = do_step(h, grad_u, grad_u, u, rows + (size_t)k * stride, (cudaStream_t)stream);
+        if (rc != TFS_OK) return rc;
+    }
+    return TFS_OK;
 }
 
 size_t tfs_halo_bytes(tfs_handle h) {
@@ -1358,16 +1468,18 @@ int tfs_bind_adjoint_workspace(tfs_handle h, void* dev_ptr, size_t bytes) {
     return TFS_OK;
 }
 
-int tfs_backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* checkpoints, int K, int steps,
-                 const void* grad_u, const void* u, double* dJ_dsigma0, double* dJ_dgrad_u, double* dJ_dWi,
-                 double* dJ_dbeta, void* stream) {
+// The reverse sweep from checkpoints (K steps apart, each segment recomputed) or
+// from the stresses of all steps (trajectory; checkpoints null, K = 0).
+static int backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* checkpoints, int K,
+                    const char* trajectory, int steps, const void* grad_u, const void* u, double* dJ_dsigma0,
+                    double* dJ_dgrad_u, double* dJ_dWi, double* dJ_dbeta, void* stream) {
     // the SDIRK2 first step's adjoint: pointwise law or implicit transport (the
     // forward refuses explicit transport with it)
     if (valid_handle(h) && h->start == TFS_START_SDIRK2 && h->explicit_transport()) return TFS_ERR_ARG;
-    if (!valid_handle(h) || !dJ_dsigma_T || !checkpoints || !grad_u || !dJ_dsigma0 || !dJ_dgrad_u || !dJ_dWi ||
+    if (!valid_handle(h) || !dJ_dsigma_T || (!checkpoints && !trajectory) || !grad_u || !dJ_dsigma0 || !dJ_dgrad_u || !dJ_dWi ||
         !dJ_dbeta)
         return TFS_ERR_ARG;
-    if (K < 1 || steps < 1) return TFS_ERR_ARG;
+    if ((checkpoints && K < 1) || steps < 1) return TFS_ERR_ARG;
     if (h->transport && !u) return TFS_ERR_ARG;
     if (!h->ws || !h->aws) return TFS_ERR_NOWORKSPACE;
     if (h->aws_bytes < adj_bytes(h, K)) return TFS_ERR_NOWORKSPACE;   // also after a change of form
@@ -1378,10 +1490,44 @@ int tfs_backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* check
     const long long blocks = (h->N + 31) / 32;
     const long long ncN = (long long)h->nc * h->N;
     cudaError_t e = cudaSuccess;
+    // the two scalars from the per-block sums; synchronises
+    auto read_scalars = [&]() -> int {
+        double out2[2] = {0.0, 0.0};
+        cudaError_t er = launch_reduce_partials(L.partials, (int)blocks, L.out2, s);
+        if (er == cudaSuccess) er = cudaMemcpyAsync(out2, L.out2, sizeof(out2), cudaMemcpyDeviceToHost, s);
+        if (er == cudaSuccess) er = cudaStreamSynchronize(s);
+        if (er != cudaSuccess) return TFS_ERR_CUDA;
+        *dJ_dWi = out2[0];
+        *dJ_dbeta = out2[1];
+        h->last_stream = s;
+        return TFS_OK;
+    };
+    for (int i = 0; i < 2 && e == cudaSuccess && h->modes_bytes() > 0; ++i) e = launch_zero(L.ell[i], h->modes_bytes(), s);
+    if (e != cudaSuccess) return TFS_ERR_CUDA;
     e = launch_zero(dJ_dsigma0, dfield, s);
     if (e == cudaSuccess) e = launch_zero(dJ_dgrad_u, (size_t)h->dim * h->dim * h->N * 8, s);
     if (e == cudaSuccess) e = launch_zero(L.partials, (size_t)blocks * 16, s);
-    for (int i = 0; i < 2 && e == cudaSuccess && h->modes_bytes() > 0; ++i) e = launch_zero(L.ell[i], h->modes_bytes(), s);
+    if (resident_path(h)) {
+        for (int end = steps; end > 0 && e == cudaSuccess;) {
+            const int start = trajectory ? 0 : (end - 1) / K * K;
+            const char* rows = trajectory;
+            size_t stride = h->field_bytes();
+            if (!trajectory) {
+                int rc = tfs_load(h, checkpoints[start / K], stream);
+                if (rc != TFS_OK) return rc;
+                if (h->step != start) return TFS_ERR_FORMAT;
+                rc = step_refused(h, grad_u, u);
+                if (rc == TFS_OK) rc = run_resident(h, end - start, grad_u, L.seg, L.seg_stride, s);
+                if (rc != TFS_OK) return rc;
+                rows = L.seg;
+                stride = L.seg_stride;
+            }
+            e = back_resident(h, start, end, grad_u, rows, stride, end == steps ? dJ_dsigma_T : nullptr, L.ell[0],
+                              L.ell[1], dJ_dsigma0, dJ_dgrad_u, L.partials, s);
+            end = start;
+        }
+        return e == cudaSuccess ? read_scalars() : TFS_ERR_CUDA;
+    }
     // J = <dJ, sigma^T>, or in the paper's variable <dJ, Psi^T> (held in lamR, the
     // adjoint of Phi^T then starts at 0)
     double* dJ_into = h->paper() ? (paper_psi_ring(h) ? L.t[0] : L.lamR) : L.s[0];
@@ -1395,7 +1541,272 @@ int tfs_backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* check
     int cur = 0;        // s[2*cur] = s1, s[2*cur+1] = s0
     int ell_prev = 0;   // slot of lamQ of the later step; the other slot holds the one before
     const LaunchCfg cfg = make_cfg(h);
-    const int nseg = (steps + K - 1) / K;
+    auto reverse_step = [&](int n, const void* sig_np1) -> int {
+        const int nxt = 1 - cur;
+        if (h->paper() && n == 0 && h->start == TFS_START_SDIRK2) {
+            // pointwise law (SDIRK2 refuses explicit transport, the adjoint implicit transport)
+            StartConsts c = start_consts(h);
+            c.g[0] = psi0_stage[0];
+            c.g[1] = psi0_stage[1];
+            const double a_p = 1.0 + h->dt * c.gam * c.W / h->Wi;
+            const double G = (1.0 - h->beta) / (h->Wi * h->Re);
+            const double* lam_psi = (steps == 1) ? L.lamR : nullptr;
+            if (h->implicit_transport()) {
+                // both stage systems global; Phi^(1) of stage 1 kept in lpp
+                int it = 0;
+                double rr = 0.0;
+                if (h->is_double()) {
+                    ImpArgs<double> ia{};
+                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                    ia.a = a_p;
+                    ia.dt = c.gam * h->dt * c.W;
+                    StartImpAdj<double> j{L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
+                                          (const double*)L.ell[1 - ell_prev], (const double*)sig_np1, L.lpp,
+                                          L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
+                                          h->Wi, h->Re, 1, lam_psi,
+                                          h->sigma0_zero ? nullptr : (const double*)h->sigma0, h->dt};
+                    e = run_start_implicit_adjoint_f64(ia, c, j, s, &it, &rr);
+                } else {
+                    ImpArgs<float> ia{};
+                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                    ia.a = a_p;
+                    ia.dt = c.gam * h->dt * c.W;
+                    StartImpAdj<float> j{L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
+                                         (const float*)L.ell[1 - ell_prev], (const float*)sig_np1, L.lpp,
+                                         L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
+                                         h->Wi, h->Re, 1, lam_psi,
+                                         h->sigma0_zero ? nullptr : (const float*)h->sigma0, h->dt};
+                    e = run_start_implicit_adjoint_f32(ia, c, j, s, &it, &rr);
+                }
+                if (e != cudaSuccess) return TFS_ERR_CUDA;
+                h->last_iters = it;
+                h->last_relres = rr;
+                cur = nxt;
+                return TFS_OK;
+            }
+            if (h->is_double()) {
+                PaperStartAdjArgs<double> a{(const double*)grad_u,
+                                            h->sigma0_zero ? nullptr : (const double*)h->sigma0, lam_psi,
+                                            L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
+                                            (const double*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
+                                            dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_p, G, h->Wi,
+                                            h->Re};
+                e = launch_paper_start_adjoint_f64(a, c, h->dim, s);
+            } else {
+                PaperStartAdjArgs<float> a{(const float*)grad_u,
+                                           h->sigma0_zero ? nullptr : (const float*)h->sigma0, lam_psi,
+                                           L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
+                                           (const float*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
+                                           dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_p, G, h->Wi,
+                                           h->Re};
+                e = launch_paper_start_adjoint_f32(a, c, h->dim, s);
+            }
+            if (e != cudaSuccess) return TFS_ERR_CUDA;
+            cur = nxt;
+            return TFS_OK;
+        }
+        if (h->paper()) {
+            const double* lam_psi = (n == steps - 1 && !paper_psi_ring(h)) ? L.lamR : nullptr;
+            if (h->implicit_transport()) {
+                // Op^T solve; the adjoint of Psi handed on carries the transport's term
+                int it = 0;
+                double rr = 0.0;
+                if (h->is_double()) {
+                    ImpArgs<double> ia{};
+                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                    fill_implicit_paper(h, ia);
+                    e = run_implicit_adjoint_f64(ia, L.s[2 * cur], (const double*)L.ell[ell_prev],
+                                                 (const double*)L.ell[1 - ell_prev], L.cfT, lam_psi, h->xi_p,
+                                                 L.lpp, s, &it, &rr);
+                } else {
+                    ImpArgs<float> ia{};
+                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                    fill_implicit_paper(h, ia);
+                    e = run_implicit_adjoint_f32(ia, L.s[2 * cur], (const float*)L.ell[ell_prev],
+                                                 (const float*)L.ell[1 - ell_prev], L.cfT, lam_psi, h->xi_p,
+                                                 L.lpp, s, &it, &rr);
+                }
+                if (e != cudaSuccess) return TFS_ERR_CUDA;
+                h->last_iters = it;
+                h->last_relres = rr;
+                lam_psi = L.lpp;
+            }
+            e = h->is_double() ? paper_adjoint_step<double>(h, L, cur, ell_prev, grad_u, u, sig_np1, lam_psi,
+                                                            psi0s[(size_t)n], dJ_dgrad_u, s)
+                               : paper_adjoint_step<float>(h, L, cur, ell_prev, grad_u, u, sig_np1, lam_psi,
+                                                           psi0s[(size_t)n], dJ_dgrad_u, s);
+            if (e != cudaSuccess) return TFS_ERR_CUDA;
+            cur = nxt;
+            ell_prev = 1 - ell_prev;
+            return TFS_OK;
+        }
+        if (n == 0 && h->start == TFS_START_SDIRK2) {
+            const StartConsts c = start_consts(h);
+            const double a_stage = h->dt * c.W + h->dt / h->Wi;
+            const double G = (1.0 - h->beta) / (h->Wi * h->Re);
+            if (h->implicit_transport()) {
+                // both stage systems are global: two transposed solves, stage 1 solved again
+                int it = 0;
+                double rr = 0.0;
+                if (h->is_double()) {
+                    ImpArgs<double> ia{};
+                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                    ia.a = a_stage;
+                    StartImpAdj<double> j{L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
+                                          (const double*)L.ell[1 - ell_prev], (const double*)sig_np1, L.lamR,
+                                          L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
+                                          h->Wi, h->Re, 0, nullptr, nullptr, h->dt};
+                    e = run_start_implicit_adjoint_f64(ia, c, j, s, &it, &rr);
+                } else {
+                    ImpArgs<float> ia{};
+                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                    ia.a = a_stage;
+                    StartImpAdj<float> j{L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
+                                         (const float*)L.ell[1 - ell_prev], (const float*)sig_np1, L.lamR,
+                                         L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
+                                         h->Wi, h->Re, 0, nullptr, nullptr, h->dt};
+                    e = run_start_implicit_adjoint_f32(ia, c, j, s, &it, &rr);
+                }
+                if (e != cudaSuccess) return TFS_ERR_CUDA;
+                h->last_iters = it;
+                h->last_relres = rr;
+                cur = nxt;
+                return TFS_OK;
+            }
+            if (h->is_double()) {
+                StartAdjArgs<double> a{(const double*)grad_u, h->sigma0_zero ? nullptr : (const double*)h->sigma0,
+                                       L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
+                                       (const double*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
+                                       dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_stage, G, h->Wi,
+                                       h->Re};
+                e = launch_start_adjoint_f64(a, c, h->dim, s);
+            } else {
+                StartAdjArgs<float> a{(const float*)grad_u, h->sigma0_zero ? nullptr : (const float*)h->sigma0,
+                                      L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
+                                      (const float*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
+                                      dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_stage, G, h->Wi,
+                                      h->Re};
+                e = launch_start_adjoint_f32(a, c, h->dim, s);
+            }
+            if (e != cudaSuccess) return TFS_ERR_CUDA;
+            cur = nxt;
+            return TFS_OK;
+        }
+        if (h->is_double()) {
+            AdjArgs<double> a{};
+            a.kap_n = (const double*)grad_u;
+            a.kap_nm1 = (const double*)grad_u;
+            a.u = (const double*)u;
+            a.sig_np1 = (const double*)sig_np1;
+            a.ell_prev = (const double*)L.ell[ell_prev];
+            a.ell_prev2 = (double*)L.ell[1 - ell_prev];
+            a.mc = h->mcd;
+            a.s1 = L.s[2 * cur];
+            a.s0 = L.s[2 * cur + 1];
+            a.s1_out = L.s[2 * nxt];
+            a.s0_out = L.s[2 * nxt + 1];
+            a.lamR = L.lamR;
+            a.g_sigma0 = dJ_dsigma0;
+            a.g_kap = dJ_dgrad_u;
+            a.partials = L.partials;
+            a.flags = h->flags;
+            a.N = h->N;
+            a.n0 = (int)h->n[0];
+            a.n1 = (int)h->n[1];
+            a.n2 = (int)h->n[2];
+            a.m = h->classic() ? 0 : h->m;
+            a.first = (n == steps - 1);
+            a.dt = h->dt;
+            a.eta = h->classic() ? kB0 : h->eta;
+            a.a = a.eta + h->dt / h->Wi;
+            a.G = (1.0 - h->beta) / (h->Wi * h->Re);
+            a.g = g_alpha(h, n);
+            a.eps = h->eps;
+            a.Wi = h->Wi;
+            a.Re = h->Re;
+            for (int i = 0; i < 3; ++i) a.inv_h[i] = (double)h->n[i] / h->L[i];
+            if (h->implicit_transport()) {
+                ImpArgs<double> ia{};
+                fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                int it = 0;
+                double rr = 0.0;
+                e = run_implicit_adjoint_f64(ia, L.s[2 * cur], a.ell_prev, a.ell_prev2, L.cfT, nullptr, 0.0,
+                                             nullptr, s, &it, &rr);
+                h->last_iters = it;
+                h->last_relres = rr;
+            }
+            if (e == cudaSuccess) e = launch_adjoint_f64(a, cfg, s);
+            if (e == cudaSuccess && h->explicit_transport()) e = launch_adjoint_transport(a, u, true, cfg, s);
+        } else {
+            AdjArgs<float> a{};
+            a.kap_n = (const float*)grad_u;
+            a.kap_nm1 = (const float*)grad_u;
+            a.u = (const float*)u;
+            a.sig_np1 = (const float*)sig_np1;
+            a.ell_prev = (const float*)L.ell[ell_prev];
+            a.ell_prev2 = (float*)L.ell[1 - ell_prev];
+            a.mc = h->mcd;
+            a.mcf = h->mcf;
+            a.s1 = L.s[2 * cur];
+            a.s0 = L.s[2 * cur + 1];
+            a.s1_out = L.s[2 * nxt];
+            a.s0_out = L.s[2 * nxt + 1];
+            a.lamR = L.lamR;
+            a.g_sigma0 = dJ_dsigma0;
+            a.g_kap = dJ_dgrad_u;
+            a.partials = L.partials;
+            a.flags = h->flags;
+            a.N = h->N;
+            a.n0 = (int)h->n[0];
+            a.n1 = (int)h->n[1];
+            a.n2 = (int)h->n[2];
+            a.m = h->classic() ? 0 : h->m;
+            a.first = (n == steps - 1);
+            a.dt = h->dt;
+            a.eta = h->classic() ? kB0 : h->eta;
+            a.a = a.eta + h->dt / h->Wi;
+            a.G = (1.0 - h->beta) / (h->Wi * h->Re);
+            a.g = g_alpha(h, n);
+            a.eps = h->eps;
+            a.Wi = h->Wi;
+            a.Re = h->Re;
+            for (int i = 0; i < 3; ++i) a.inv_h[i] = (double)h->n[i] / h->L[i];
+            if (h->implicit_transport()) {
+                ImpArgs<float> ia{};
+                fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
+                int it = 0;
+                double rr = 0.0;
+                e = run_implicit_adjoint_f32(ia, L.s[2 * cur], a.ell_prev, a.ell_prev2, L.cfT, nullptr, 0.0,
+                                             nullptr, s, &it, &rr);
+                h->last_iters = it;
+                h->last_relres = rr;
+            }
+            if (e == cudaSuccess) e = launch_adjoint_f32(a, cfg, s);
+            if (e == cudaSuccess && h->explicit_transport()) {
+                AdjArgs<double> ad{};
+                ad.N = a.N;
+                ad.n0 = a.n0;
+                ad.n1 = a.n1;
+                ad.n2 = a.n2;
+                ad.dt = a.dt;
+                ad.eps = a.eps;
+                for (int i = 0; i < 3; ++i) ad.inv_h[i] = a.inv_h[i];
+                ad.lamR = a.lamR;
+                ad.s1_out = a.s1_out;
+                ad.s0_out = a.s0_out;
+                e = launch_adjoint_transport(ad, u, false, cfg, s);
+            }
+        }
+        if (e != cudaSuccess) return TFS_ERR_CUDA;
+        cur = nxt;
+        if (!h->classic()) ell_prev = 1 - ell_prev;
+        return TFS_OK;
+    };
+    for (int n = steps - 1; n >= 0 && trajectory; --n) {
+        const int rc = reverse_step(n, trajectory + (size_t)n * h->field_bytes());
+        if (rc != TFS_OK) return rc;
+    }
+    const int nseg = trajectory ? 0 : (steps + K - 1) / K;
     for (int seg = nseg - 1; seg >= 0; --seg) {
         const int start = seg * K;
         const int end = (start + K < steps) ? start + K : steps;
@@ -1407,278 +1818,31 @@ int tfs_backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* check
             if (rc != TFS_OK) return rc;
         }
         for (int n = end - 1; n >= start; --n) {
-            const void* sig_np1 = L.seg + (size_t)(n - start) * L.seg_stride;
-            const int nxt = 1 - cur;
-            if (h->paper() && n == 0 && h->start == TFS_START_SDIRK2) {
-                // pointwise law (SDIRK2 refuses explicit transport, the adjoint implicit transport)
-                StartConsts c = start_consts(h);
-                c.g[0] = psi0_stage[0];
-                c.g[1] = psi0_stage[1];
-                const double a_p = 1.0 + h->dt * c.gam * c.W / h->Wi;
-                const double G = (1.0 - h->beta) / (h->Wi * h->Re);
-                const double* lam_psi = (steps == 1) ? L.lamR : nullptr;
-                if (h->implicit_transport()) {
-                    // both stage systems global; Phi^(1) of stage 1 kept in lpp
-                    int it = 0;
-                    double rr = 0.0;
-                    if (h->is_double()) {
-                        ImpArgs<double> ia{};
-                        fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                        ia.a = a_p;
-                        ia.dt = c.gam * h->dt * c.W;
-                        StartImpAdj<double> j{L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
-                                              (const double*)L.ell[1 - ell_prev], (const double*)sig_np1, L.lpp,
-                                              L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
-                                              h->Wi, h->Re, 1, lam_psi,
-                                              h->sigma0_zero ? nullptr : (const double*)h->sigma0, h->dt};
-                        e = run_start_implicit_adjoint_f64(ia, c, j, s, &it, &rr);
-                    } else {
-                        ImpArgs<float> ia{};
-                        fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                        ia.a = a_p;
-                        ia.dt = c.gam * h->dt * c.W;
-                        StartImpAdj<float> j{L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
-                                             (const float*)L.ell[1 - ell_prev], (const float*)sig_np1, L.lpp,
-                                             L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
-                                             h->Wi, h->Re, 1, lam_psi,
-                                             h->sigma0_zero ? nullptr : (const float*)h->sigma0, h->dt};
-                        e = run_start_implicit_adjoint_f32(ia, c, j, s, &it, &rr);
-                    }
-                    if (e != cudaSuccess) return TFS_ERR_CUDA;
-                    h->last_iters = it;
-                    h->last_relres = rr;
-                    cur = nxt;
-                    continue;
-                }
-                if (h->is_double()) {
-                    PaperStartAdjArgs<double> a{(const double*)grad_u,
-                                                h->sigma0_zero ? nullptr : (const double*)h->sigma0, lam_psi,
-                                                L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
-                                                (const double*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
-                                                dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_p, G, h->Wi,
-                                                h->Re};
-                    e = launch_paper_start_adjoint_f64(a, c, h->dim, s);
-                } else {
-                    PaperStartAdjArgs<float> a{(const float*)grad_u,
-                                               h->sigma0_zero ? nullptr : (const float*)h->sigma0, lam_psi,
-                                               L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
-                                               (const float*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
-                                               dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_p, G, h->Wi,
-                                               h->Re};
-                    e = launch_paper_start_adjoint_f32(a, c, h->dim, s);
-                }
-                if (e != cudaSuccess) return TFS_ERR_CUDA;
-                cur = nxt;
-                continue;
-            }
-            if (h->paper()) {
-                const double* lam_psi = (n == steps - 1 && !paper_psi_ring(h)) ? L.lamR : nullptr;
-                if (h->implicit_transport()) {
-                    // Op^T solve; the adjoint of Psi handed on carries the transport's term
-                    int it = 0;
-                    double rr = 0.0;
-                    if (h->is_double()) {
-                        ImpArgs<double> ia{};
-                        fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                        fill_implicit_paper(h, ia);
-                        e = run_implicit_adjoint_f64(ia, L.s[2 * cur], (const double*)L.ell[ell_prev],
-                                                     (const double*)L.ell[1 - ell_prev], L.cfT, lam_psi, h->xi_p,
-                                                     L.lpp, s, &it, &rr);
-                    } else {
-                        ImpArgs<float> ia{};
-                        fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                        fill_implicit_paper(h, ia);
-                        e = run_implicit_adjoint_f32(ia, L.s[2 * cur], (const float*)L.ell[ell_prev],
-                                                     (const float*)L.ell[1 - ell_prev], L.cfT, lam_psi, h->xi_p,
-                                                     L.lpp, s, &it, &rr);
-                    }
-                    if (e != cudaSuccess) return TFS_ERR_CUDA;
-                    h->last_iters = it;
-                    h->last_relres = rr;
-                    lam_psi = L.lpp;
-                }
-                e = h->is_double() ? paper_adjoint_step<double>(h, L, cur, ell_prev, grad_u, u, sig_np1, lam_psi,
-                                                                psi0s[(size_t)n], dJ_dgrad_u, s)
-                                   : paper_adjoint_step<float>(h, L, cur, ell_prev, grad_u, u, sig_np1, lam_psi,
-                                                               psi0s[(size_t)n], dJ_dgrad_u, s);
-                if (e != cudaSuccess) return TFS_ERR_CUDA;
-                cur = nxt;
-                ell_prev = 1 - ell_prev;
-                continue;
-            }
-            if (n == 0 && h->start == TFS_START_SDIRK2) {
-                const StartConsts c = start_consts(h);
-                const double a_stage = h->dt * c.W + h->dt / h->Wi;
-                const double G = (1.0 - h->beta) / (h->Wi * h->Re);
-                if (h->implicit_transport()) {
-                    // both stage systems are global: two transposed solves, stage 1 solved again
-                    int it = 0;
-                    double rr = 0.0;
-                    if (h->is_double()) {
-                        ImpArgs<double> ia{};
-                        fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                        ia.a = a_stage;
-                        StartImpAdj<double> j{L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
-                                              (const double*)L.ell[1 - ell_prev], (const double*)sig_np1, L.lamR,
-                                              L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
-                                              h->Wi, h->Re, 0, nullptr, nullptr, h->dt};
-                        e = run_start_implicit_adjoint_f64(ia, c, j, s, &it, &rr);
-                    } else {
-                        ImpArgs<float> ia{};
-                        fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                        ia.a = a_stage;
-                        StartImpAdj<float> j{L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
-                                             (const float*)L.ell[1 - ell_prev], (const float*)sig_np1, L.lamR,
-                                             L.s[2 * nxt], L.s[2 * nxt + 1], dJ_dgrad_u, L.partials, L.cfT,
-                                             h->Wi, h->Re, 0, nullptr, nullptr, h->dt};
-                        e = run_start_implicit_adjoint_f32(ia, c, j, s, &it, &rr);
-                    }
-                    if (e != cudaSuccess) return TFS_ERR_CUDA;
-                    h->last_iters = it;
-                    h->last_relres = rr;
-                    cur = nxt;
-                    continue;
-                }
-                if (h->is_double()) {
-                    StartAdjArgs<double> a{(const double*)grad_u, h->sigma0_zero ? nullptr : (const double*)h->sigma0,
-                                           L.s[2 * cur], L.s[2 * cur + 1], (const double*)L.ell[ell_prev],
-                                           (const double*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
-                                           dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_stage, G, h->Wi,
-                                           h->Re};
-                    e = launch_start_adjoint_f64(a, c, h->dim, s);
-                } else {
-                    StartAdjArgs<float> a{(const float*)grad_u, h->sigma0_zero ? nullptr : (const float*)h->sigma0,
-                                          L.s[2 * cur], L.s[2 * cur + 1], (const float*)L.ell[ell_prev],
-                                          (const float*)L.ell[1 - ell_prev], L.s[2 * nxt], L.s[2 * nxt + 1],
-                                          dJ_dgrad_u, L.partials, h->flags, h->N, h->m, h->dt, a_stage, G, h->Wi,
-                                          h->Re};
-                    e = launch_start_adjoint_f32(a, c, h->dim, s);
-                }
-                if (e != cudaSuccess) return TFS_ERR_CUDA;
-                cur = nxt;
-                continue;
-            }
-            if (h->is_double()) {
-                AdjArgs<double> a{};
-                a.kap_n = (const double*)grad_u;
-                a.kap_nm1 = (const double*)grad_u;
-                a.u = (const double*)u;
-                a.sig_np1 = (const double*)sig_np1;
-                a.ell_prev = (const double*)L.ell[ell_prev];
-                a.ell_prev2 = (double*)L.ell[1 - ell_prev];
-                a.mc = h->mcd;
-                a.s1 = L.s[2 * cur];
-                a.s0 = L.s[2 * cur + 1];
-                a.s1_out = L.s[2 * nxt];
-                a.s0_out = L.s[2 * nxt + 1];
-                a.lamR = L.lamR;
-                a.g_sigma0 = dJ_dsigma0;
-                a.g_kap = dJ_dgrad_u;
-                a.partials = L.partials;
-                a.flags = h->flags;
-                a.N = h->N;
-                a.n0 = (int)h->n[0];
-                a.n1 = (int)h->n[1];
-                a.n2 = (int)h->n[2];
-                a.m = h->classic() ? 0 : h->m;
-                a.first = (n == steps - 1);
-                a.dt = h->dt;
-                a.eta = h->classic() ? kB0 : h->eta;
-                a.a = a.eta + h->dt / h->Wi;
-                a.G = (1.0 - h->beta) / (h->Wi * h->Re);
-                a.g = g_alpha(h, n);
-                a.eps = h->eps;
-                a.Wi = h->Wi;
-                a.Re = h->Re;
-                for (int i = 0; i < 3; ++i) a.inv_h[i] = (double)h->n[i] / h->L[i];
-                if (h->implicit_transport()) {
-                    ImpArgs<double> ia{};
-                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                    int it = 0;
-                    double rr = 0.0;
-                    e = run_implicit_adjoint_f64(ia, L.s[2 * cur], a.ell_prev, a.ell_prev2, L.cfT, nullptr, 0.0,
-                                                 nullptr, s, &it, &rr);
-                    h->last_iters = it;
-                    h->last_relres = rr;
-                }
-                if (e == cudaSuccess) e = launch_adjoint_f64(a, cfg, s);
-                if (e == cudaSuccess && h->explicit_transport()) e = launch_adjoint_transport(a, u, true, cfg, s);
-            } else {
-                AdjArgs<float> a{};
-                a.kap_n = (const float*)grad_u;
-                a.kap_nm1 = (const float*)grad_u;
-                a.u = (const float*)u;
-                a.sig_np1 = (const float*)sig_np1;
-                a.ell_prev = (const float*)L.ell[ell_prev];
-                a.ell_prev2 = (float*)L.ell[1 - ell_prev];
-                a.mc = h->mcd;
-                a.mcf = h->mcf;
-                a.s1 = L.s[2 * cur];
-                a.s0 = L.s[2 * cur + 1];
-                a.s1_out = L.s[2 * nxt];
-                a.s0_out = L.s[2 * nxt + 1];
-                a.lamR = L.lamR;
-                a.g_sigma0 = dJ_dsigma0;
-                a.g_kap = dJ_dgrad_u;
-                a.partials = L.partials;
-                a.flags = h->flags;
-                a.N = h->N;
-                a.n0 = (int)h->n[0];
-                a.n1 = (int)h->n[1];
-                a.n2 = (int)h->n[2];
-                a.m = h->classic() ? 0 : h->m;
-                a.first = (n == steps - 1);
-                a.dt = h->dt;
-                a.eta = h->classic() ? kB0 : h->eta;
-                a.a = a.eta + h->dt / h->Wi;
-                a.G = (1.0 - h->beta) / (h->Wi * h->Re);
-                a.g = g_alpha(h, n);
-                a.eps = h->eps;
-                a.Wi = h->Wi;
-                a.Re = h->Re;
-                for (int i = 0; i < 3; ++i) a.inv_h[i] = (double)h->n[i] / h->L[i];
-                if (h->implicit_transport()) {
-                    ImpArgs<float> ia{};
-                    fill_implicit(h, ia, grad_u, grad_u, u, nullptr, h->third_sig(), h->cur_mode, 1 - h->cur_mode);
-                    int it = 0;
-                    double rr = 0.0;
-                    e = run_implicit_adjoint_f32(ia, L.s[2 * cur], a.ell_prev, a.ell_prev2, L.cfT, nullptr, 0.0,
-                                                 nullptr, s, &it, &rr);
-                    h->last_iters = it;
-                    h->last_relres = rr;
-                }
-                if (e == cudaSuccess) e = launch_adjoint_f32(a, cfg, s);
-                if (e == cudaSuccess && h->explicit_transport()) {
-                    AdjArgs<double> ad{};
-                    ad.N = a.N;
-                    ad.n0 = a.n0;
-                    ad.n1 = a.n1;
-                    ad.n2 = a.n2;
-                    ad.dt = a.dt;
-                    ad.eps = a.eps;
-                    for (int i = 0; i < 3; ++i) ad.inv_h[i] = a.inv_h[i];
-                    ad.lamR = a.lamR;
-                    ad.s1_out = a.s1_out;
-                    ad.s0_out = a.s0_out;
-                    e = launch_adjoint_transport(ad, u, false, cfg, s);
-                }
-            }
-            if (e != cudaSuccess) return TFS_ERR_CUDA;
-            cur = nxt;
-            if (!h->classic()) ell_prev = 1 - ell_prev;
+            rc = reverse_step(n, L.seg + (size_t)(n - start) * L.seg_stride);
+            if (rc != TFS_OK) return rc;
         }
     }
     // initial state sigma^0 = sigma^{-1} = sigma0
     e = launch_add_initial(dJ_dsigma0, L.s[2 * cur], L.s[2 * cur + 1], ncN, s);
-    if (e == cudaSuccess) e = launch_reduce_partials(L.partials, (int)blocks, L.out2, s);
-    double out2[2] = {0.0, 0.0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out2, L.out2, sizeof(out2), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return TFS_ERR_CUDA;
-    *dJ_dWi = out2[0];
-    *dJ_dbeta = out2[1];
-    h->last_stream = s;
-    return TFS_OK;
+    return e == cudaSuccess ? read_scalars() : TFS_ERR_CUDA;
+}
+
+int tfs_backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* checkpoints, int K, int steps,
+                 const void* grad_u, const void* u, double* dJ_dsigma0, double* dJ_dgrad_u, double* dJ_dWi,
+                 double* dJ_dbeta, void* stream) {
+    if (!checkpoints) return TFS_ERR_ARG;
+    return backward(h, dJ_dsigma_T, checkpoints, K, nullptr, steps, grad_u, u, dJ_dsigma0, dJ_dgrad_u, dJ_dWi, dJ_dbeta,
+                    stream);
+}
+
+int tfs_backward_run(tfs_handle h, const void* dJ_dsigma_T, const void* trajectory, int steps, const void* grad_u,
+                     const void* u, double* dJ_dsigma0, double* dJ_dgrad_u, double* dJ_dWi, double* dJ_dbeta,
+                     void* stream) {
+    if (!valid_handle(h) || !trajectory || ((uintptr_t)trajectory) % 16) return TFS_ERR_ARG;
+    // these reverse steps solve the run's global systems again from its state
+    if (h->start == TFS_START_SDIRK2 || h->implicit_transport()) return TFS_ERR_ARG;
+    return backward(h, dJ_dsigma_T, nullptr, 0, (const char*)trajectory, steps, grad_u, u, dJ_dsigma0, dJ_dgrad_u,
+                    dJ_dWi, dJ_dbeta, stream);
 }
 
 int tfs_status(tfs_handle h, unsigned* device_flags) {

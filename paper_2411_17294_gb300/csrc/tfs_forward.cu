@@ -265,90 +265,6 @@ __device__ __forceinline__ T finish_stencil(const FwdArgs<T>& A, int stencil, co
     return (T)A.dt * adv - (T)(A.eps * A.dt) * lap;
 }
 
-// ----------------------------------------------------------- FP32 point solve
-// Packed residual r = R - a x + dt (K x + x K^T) with R, a, dt, K as double-float
-// and x a float vector.  R - a x is formed exactly (TwoProd); the operator term
-// is a compensated dot product (Ogita-Rump-Oishi Dot2) of the K entries with x.
-template <int DIM>
-__device__ __forceinline__ void residual_f2(const f2 K[3][3], F2c a, F2c dt, const f2 R[Packed<DIM>::NC],
-                                            const float x[Packed<DIM>::NC], f2 r[Packed<DIM>::NC]) {
-    constexpr int NC = Packed<DIM>::NC;
-    float S[3][3];
-    static_for<0, NC>([&](auto cc) {
-        constexpr int c = decltype(cc)::value;
-        S[Packed<DIM>::I(c)][Packed<DIM>::J(c)] = x[c];
-        S[Packed<DIM>::J(c)][Packed<DIM>::I(c)] = x[c];
-    });
-    const f2 dtf{dt.hi, dt.lo};
-    static_for<0, NC>([&](auto cc) {
-        constexpr int c = decltype(cc)::value;
-        constexpr int i = Packed<DIM>::I(c), j = Packed<DIM>::J(c);
-        float bs = 0.0f, be = 0.0f;
-        auto term = [&](const f2 k, float v) {
-            const f2 pr = two_prod(k.hi, v);
-            const f2 sm = two_sum_f2(bs, pr.hi);
-            bs = sm.hi;
-            be = __fadd_rn(be, __fadd_rn(sm.lo, __fmaf_rn(k.lo, v, pr.lo)));
-        };
-        static_for<0, DIM>([&](auto ll) {
-            constexpr int l = decltype(ll)::value;
-            term(K[i][l], S[l][j]);
-            term(K[j][l], S[i][l]);
-        });
-        const f2 ax = [&] {
-            f2 pr = two_prod(a.hi, x[c]);
-            pr.lo = __fmaf_rn(a.lo, x[c], pr.lo);
-            return pr;
-        }();
-        const f2 t = f2_add(R[c], f2_neg(ax));
-        r[c] = f2_add(t, f2_mul(dtf, fast_two_sum(bs, be)));
-    });
-}
-
-template <int DIM>
-__device__ __forceinline__ bool solve_point_f32(const f2 K[3][3], F2c a, F2c dt, const f2 R[Packed<DIM>::NC],
-                                                f2 x[Packed<DIM>::NC]) {
-    constexpr int NC = Packed<DIM>::NC;
-    LU32<NC> F;
-    const float af = a.hi, dtf = dt.hi;
-    static_for<0, NC>([&](auto rr) {
-        constexpr int r = decltype(rr)::value;
-        static_for<0, NC>([&](auto kk) {
-            constexpr int k = decltype(kk)::value;
-            constexpr int ro = Packed<DIM>::I(r), so = Packed<DIM>::J(r);
-            constexpr int i = Packed<DIM>::I(k), j = Packed<DIM>::J(k);
-            float v = 0.0f;
-            if (so == j) v += K[ro][i].hi;
-            if (i != j && so == i) v += K[ro][j].hi;
-            if (ro == i) v += K[so][j].hi;
-            if (i != j && ro == j) v += K[so][i].hi;
-            F.a[r][k] = (r == k) ? __fmaf_rn(-dtf, v, af) : -dtf * v;
-        });
-    });
-    // row diagonal dominance (the usual case: a = eta + dt/Wi against dt |kappa*|)
-    // allows elimination without row exchanges; otherwise partial pivoting
-    const bool ok = row_dominant<NC>(F) ? lu32_factor_nopivot<NC>(F, 1e-30f) : lu32_factor<NC>(F, 1e-30f);
-    float x0[NC];
-    static_for<0, NC>([&](auto rr) {
-        constexpr int r = decltype(rr)::value;
-        x0[r] = R[r].hi + R[r].lo;
-    });
-    lu32_solve<NC>(F, x0);
-    f2 res[NC];
-    residual_f2<DIM>(K, a, dt, R, x0, res);
-    float d[NC];
-    static_for<0, NC>([&](auto rr) {
-        constexpr int r = decltype(rr)::value;
-        d[r] = res[r].hi + res[r].lo;
-    });
-    lu32_solve<NC>(F, d);
-    static_for<0, NC>([&](auto rr) {
-        constexpr int r = decltype(rr)::value;
-        x[r] = two_sum_f2(x0[r], d[r]);
-    });
-    return ok;
-}
-
 // ----------------------------------------------------------------- the kernels
 // Transport pre-pass: A_c(p) = dt sum_a u_a D_a(E_c) - eps dt Lap(E_c) for all
 // components at point p (one thread per point), and the Courant flag.

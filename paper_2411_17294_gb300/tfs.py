@@ -28,8 +28,8 @@ TFS_FLAG_NONFINITE, TFS_FLAG_SINGULAR, TFS_FLAG_COURANT, TFS_FLAG_TIMEOUT, TFS_F
 
 EXPORTS = [
     "tfs_create", "tfs_set_param", "tfs_set_soe", "tfs_transport_limit", "tfs_workspace_bytes", "tfs_bind_workspace",
-    "tfs_set_state", "tfs_step", "tfs_get_stress", "tfs_set_step_events", "tfs_step_index", "tfs_last_solve", "tfs_checkpoint_bytes", "tfs_save",
-    "tfs_load", "tfs_adjoint_workspace_bytes", "tfs_bind_adjoint_workspace", "tfs_backward", "tfs_status",
+    "tfs_set_state", "tfs_step", "tfs_run", "tfs_get_stress", "tfs_set_step_events", "tfs_step_index", "tfs_last_solve", "tfs_checkpoint_bytes", "tfs_save",
+    "tfs_load", "tfs_adjoint_workspace_bytes", "tfs_bind_adjoint_workspace", "tfs_backward", "tfs_backward_run", "tfs_status",
     "tfs_strerror", "tfs_destroy", "tfs_run_static", "tfs_static_status", "tfs_check_wait_bound",
     "tfs_halo_bytes", "tfs_get_halo", "tfs_step_slab",
     "tfs_ns_create", "tfs_ns_workspace_bytes", "tfs_ns_bind_workspace", "tfs_ns_set_state", "tfs_ns_step",
@@ -71,6 +71,7 @@ def load_library(path: str | None = None):
         "tfs_bind_workspace": (ctypes.c_int, [H, vp, sz]),
         "tfs_set_state": (ctypes.c_int, [H, vp, vp]),
         "tfs_step": (ctypes.c_int, [H, vp, vp, vp, vp]),
+        "tfs_run": (ctypes.c_int, [H, ctypes.c_int, vp, vp, vp, vp]),
         "tfs_get_stress": (ctypes.c_int, [H, vp, vp]),
         "tfs_set_step_events": (ctypes.c_int, [H, vp, vp]),
         "tfs_step_index": (ctypes.c_long, [H]),
@@ -82,6 +83,7 @@ def load_library(path: str | None = None):
         "tfs_bind_adjoint_workspace": (ctypes.c_int, [H, vp, sz]),
         "tfs_backward": (ctypes.c_int, [H, vp, ctypes.POINTER(vp), ctypes.c_int, ctypes.c_int, vp, vp, vp, vp,
                                         dp, dp, vp]),
+        "tfs_backward_run": (ctypes.c_int, [H, vp, vp, ctypes.c_int, vp, vp, vp, vp, dp, dp, vp]),
         "tfs_status": (ctypes.c_int, [H, ctypes.POINTER(ctypes.c_uint)]),
         "tfs_strerror": (ctypes.c_char_p, [ctypes.c_int]),
         "tfs_destroy": (ctypes.c_int, [H]),
@@ -242,6 +244,19 @@ class Solver:
         check(self.lib.tfs_step(self.h, ctypes.c_void_p(kn), ctypes.c_void_p(knm1), ctypes.c_void_p(up),
                                 ctypes.c_void_p(_stream_ptr(stream))), "tfs_step")
 
+    def run(self, steps: int, grad_u, u=None, stream=None):
+        """`steps` steps with the frozen grad_u (tfs_run); returns the stress
+        after each step, [steps, nc, N].  Tensors as for step()."""
+        torch = _torch()
+        traj = torch.empty((int(steps), self.nc, self.N), dtype=self.dtype, device=self.device)
+        if stream is not None:
+            traj.record_stream(stream)
+        check(self.lib.tfs_run(self.h, int(steps), ctypes.c_void_p(grad_u.data_ptr()),
+                               ctypes.c_void_p(u.data_ptr() if u is not None else 0),
+                               ctypes.c_void_p(traj.data_ptr()),
+                               ctypes.c_void_p(_stream_ptr(stream))), "tfs_run")
+        return traj
+
     def halo_buffers(self):
         """Two halo buffers (lo, hi) for a slab of this handle's grid:
         [2 levels][nc][2 planes][plane points] tensors of the handle's dtype."""
@@ -337,14 +352,9 @@ class Solver:
     def backward(self, dJ_dsigma_T, checkpoints, K: int, steps: int, grad_u, u=None, stream=None):
         """Gradients of J for a frozen-gradient run of `steps` steps; returns
         (dJ/dsigma0 [nc,N] f64, dJ/dgrad_u [d*d,N] f64, dJ/dWi, dJ/dbeta)."""
-        torch = _torch()
         self.ensure_adjoint_workspace(K)
-        g_s0 = torch.empty((self.nc, self.N), dtype=torch.float64, device=self.device)
-        g_k = torch.empty((self.dim * self.dim, self.N), dtype=torch.float64, device=self.device)
-        dJ = self._field(dJ_dsigma_T, self.nc)
+        g_s0, g_k, dJ, gWi, gb = self._gradient_buffers(dJ_dsigma_T)
         arr = (ctypes.c_void_p * len(checkpoints))(*[ctypes.c_void_p(c.data_ptr()) for c in checkpoints])
-        gWi = ctypes.c_double(0.0)
-        gb = ctypes.c_double(0.0)
         check(self.lib.tfs_backward(self.h, ctypes.c_void_p(dJ.data_ptr()), arr, int(K), int(steps),
                                     ctypes.c_void_p(grad_u.data_ptr()),
                                     ctypes.c_void_p(u.data_ptr() if u is not None else 0),
@@ -352,6 +362,25 @@ class Solver:
                                     ctypes.byref(gWi), ctypes.byref(gb), ctypes.c_void_p(_stream_ptr(stream))),
               "tfs_backward")
         return g_s0, g_k, gWi.value, gb.value
+
+    def backward_run(self, dJ_dsigma_T, trajectory, grad_u, u=None, stream=None):
+        """backward() from the trajectory that run() returned for all steps
+        since set_state (nothing is recomputed)."""
+        self.ensure_adjoint_workspace(1)
+        g_s0, g_k, dJ, gWi, gb = self._gradient_buffers(dJ_dsigma_T)
+        check(self.lib.tfs_backward_run(self.h, ctypes.c_void_p(dJ.data_ptr()), ctypes.c_void_p(trajectory.data_ptr()),
+                                        int(trajectory.shape[0]), ctypes.c_void_p(grad_u.data_ptr()),
+                                        ctypes.c_void_p(u.data_ptr() if u is not None else 0),
+                                        ctypes.c_void_p(g_s0.data_ptr()), ctypes.c_void_p(g_k.data_ptr()),
+                                        ctypes.byref(gWi), ctypes.byref(gb), ctypes.c_void_p(_stream_ptr(stream))),
+              "tfs_backward_run")
+        return g_s0, g_k, gWi.value, gb.value
+
+    def _gradient_buffers(self, dJ_dsigma_T):
+        torch = _torch()
+        return (torch.empty((self.nc, self.N), dtype=torch.float64, device=self.device),
+                torch.empty((self.dim * self.dim, self.N), dtype=torch.float64, device=self.device),
+                self._field(dJ_dsigma_T, self.nc), ctypes.c_double(0.0), ctypes.c_double(0.0))
 
     def close(self):
         if getattr(self, "h", None) is not None and self.h.value:

@@ -412,8 +412,8 @@ typedef struct tfs_ns_ctx* tfs_ns_handle;
 int tfs_ns_create(tfs_ns_handle* h, int n0, int n1, double L0, double L1, double beta, double Re, double dt,
                   int precision);
 
-/* Device workspace of the handle: 21 complex and 8 real FP64 fields of n0 n1
-   values and the transforms' twiddle tables (n0/2 + n1/2 complex), each
+/* Device workspace of the handle: 14 complex and 6 real FP64 fields of n0 n1
+   values and the transforms' twiddle tables (n0 + n1 complex), each
    rounded up to 256 bytes. */
 size_t tfs_ns_workspace_bytes(tfs_ns_handle h);
 

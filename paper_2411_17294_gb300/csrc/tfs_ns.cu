@@ -15,10 +15,23 @@
 // the grid.  The transforms are this file's own: a Stockham autosort FFT of
 // each row in shared memory (the formulation of Govindaraju et al.,
 // "High performance discrete Fourier transforms on graphics processors",
-// SC 2008) in radix 4, FP64 complex, and a tiled transpose between the two axes; spectral
-// arrays are kept transposed, [kx][ky].  Real fields go two to a complex
-// transform (f + i g forward, split by the Hermitian symmetry of real spectra;
-// A + i B inverse), so a step takes 6 two-dimensional transforms, not 11.
+// SC 2008) in radix 4, FP64 complex; spectral arrays are kept transposed, [kx][ky].
+//
+// Bound: the FP64 pipe (2 operations per clock and SM); a row pass over 1024^2 points is
+// 33.5 M FP64 operations, 57 us of it.  So the step is arranged to transform
+// and to compute as little as possible:
+//   - real fields go two to a complex transform (f + i g forward, split by the
+//     Hermitian symmetry of real spectra; A + i B inverse);
+//   - of the stress only xx - yy and xy are transformed: an isotropic part adds
+//     a gradient to the explicit terms, which the projection removes, so a step
+//     takes 5 two-dimensional transforms (convection 1, stress 1, velocity 1, gradient 2);
+//   - one kernel per mode goes from the two forward transforms to the three
+//     inverse ones (splitting, divergence, Helmholtz update, gradient, packing);
+//   - products, packing and rounding happen where the row passes load and store,
+//     and a pass whose rows become columns next writes them transposed.
+// Six launches per step.  Measured per step (FP32 exchange, CUDA events): 1024^2 1.40 -> 0.92 ms (a row
+// pass 73 - 86 us, was 83 and its transposes, packing and splitting apart; the kernel per mode 150 us, was
+// 153 and 125 in four others), 128^2 49 us.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -41,106 +54,158 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
+// conjugate, on the integer pipe
+__device__ __forceinline__ double2 conj_of(double2 a) {
+    return make_double2(a.x, __longlong_as_double(__double_as_longlong(a.y) ^ (long long)0x8000000000000000ull));
+}
 // i d a for a real d (the first-derivative multiplier)
 __device__ __forceinline__ double2 cimul(double d, double2 a) { return make_double2(-d * a.y, d * a.x); }
 
+// What a row pass reads: complex rows, two real fields as f + i g (g absent: 0),
+// the stress as (xx - yy) + i xy, or the convective term of the grid fields
+// u [2][N] and kap [4][N], (u.grad)u_x + i (u.grad)u_y.
+enum { kLoadComplex, kLoadPair, kLoadStress, kLoadConvection };
+// What it writes: complex rows, complex rows transposed (out[c][r]), or the real
+// and imaginary parts as real fields (FP64 and the caller's type, each when given).
+enum { kStoreRows, kStoreTransposed, kStoreFields };
+
+template <typename T>
+struct RowPass {
+    const double2* in[3];      // one per blockIdx.y
+    double2* out[3];
+    const T *f, *g;            // kLoadPair, kLoadStress (f: packed xx, xy, yy)
+    const double *u, *kap;     // kLoadConvection
+    double *da[3], *db[3];     // kStoreFields
+    T *ta[3], *tb[3];
+    int n, rows, per_block;    // row length, rows, rows per block
+    const double2* tw;
+    int inverse;
+    long long N;
+};
+
+// Points a block transforms at most (measured at 1024^2: 925 us per step against 974 with 2048, whose
+// 512 blocks of a pass leave an SM's last wave nearly empty), and blocks a pass should have at
+// least: shorter rows go one to a block on small grids.
+constexpr int kRowElems = 1024;
+constexpr int kRowBlocks = 152;
+
 // DFT of each row of length n (a power of two, 2 .. kMaxLen) with
-// exp(-+ 2 pi i j k / n) (forward / inverse), times `scale`; one block per row,
-// rows of `in` and `out` n elements apart (in == out allowed: a row is read
-// whole first).  tw[t] = exp(-2 pi i t / n), t < n (computed once on the host
+// exp(-+ 2 pi i j k / n) (forward / inverse), unscaled; a block takes per_block
+// rows.  tw[t] = exp(-2 pi i t / n), t < n (computed once on the host
 // in FP64).  Stockham autosort, radix 4: stage Ns = 1, 4, 16, ... takes the
 // four operands j + r n/4 (r = 0..3) of butterfly j, turns operand r by
 // exp(-+ 2 pi i r k / (4 Ns)) = tw[r k n / (4 Ns)], k = j mod Ns, applies the
 // 4-point DFT and writes output r to (j / Ns) 4 Ns + k + r Ns; a length that is
-// not a power of four ends with one radix-2 stage (Ns = n/2).  The buffers
-// ping-pong in shared memory; the result is in natural order.
-__global__ void __launch_bounds__(kNsThreads) fft_rows_kernel(const double2* in, double2* out, int n,
-                                                              const double2* __restrict__ tw, int inverse,
-                                                              double scale) {
+// not a power of four ends with one radix-2 stage (Ns = n/2).  A stage holds its butterflies in
+// registers between reading and writing the one shared buffer, whose
+// rows are n + 1 apart (the transposed store then reads different banks).
+// Several blocks per SM and more than one wave of them, so that the loads and
+// stores of some run beside the arithmetic of others.
+template <typename T, int LOAD, int STORE>
+__global__ void __launch_bounds__(kNsThreads, 5) fft_pass_kernel(const RowPass<T> A) {
     extern __shared__ double2 fft_buf[];
-    double2* x = fft_buf;
-    double2* y = fft_buf + n;
-    const double2* src = in + (long long)blockIdx.x * n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = src[i];
+    const int n = A.n, R = A.per_block, ld = n + 1;
+    const int which = blockIdx.y;
+    const int r0 = blockIdx.x * R;
+    const int tid = threadIdx.x;
+    const int count = R * n;
+    const int lg = 31 - __clz(n);
+    for (int e = tid; e < count; e += kNsThreads) {
+        const int r = e >> lg, c = e & (n - 1);
+        const long long q = ((long long)(r0 + r) << lg) + c;
+        double2 v;
+        if (LOAD == kLoadComplex) v = A.in[which][q];
+        else if (LOAD == kLoadPair) v = make_double2((double)A.f[q], A.g ? (double)A.g[q] : 0.0);
+        else if (LOAD == kLoadStress) v = make_double2((double)A.f[q] - (double)A.f[2 * A.N + q], (double)A.f[A.N + q]);
+        else {
+            const double ux = A.u[q], uy = A.u[A.N + q];
+            v = make_double2(ux * A.kap[q] + uy * A.kap[A.N + q], ux * A.kap[2 * A.N + q] + uy * A.kap[3 * A.N + q]);
+        }
+        fft_buf[r * ld + c] = v;
+    }
     __syncthreads();
     const int quarter = n >> 2;
+    const bool inverse = A.inverse != 0;
+    constexpr int kMine = kRowElems / 4 / kNsThreads;   // butterflies of a thread, held in registers
     int ns = 1;
     for (; 4 * ns <= n; ns <<= 2) {
-        const int step = n / (4 * ns);
-        for (int j = threadIdx.x; j < quarter; j += blockDim.x) {
-            const int k = j & (ns - 1);
+        const int step = n / (4 * ns), lq = lg - 2;
+        double2 o[kMine][4];
+#pragma unroll
+        for (int i = 0; i < kMine; ++i) {
+            const int b = tid + i * kNsThreads;
+            if (b >= R * quarter) continue;
+            const int j = b & (quarter - 1), k = j & (ns - 1);
+            const double2* x = fft_buf + (b >> lq) * ld;
             const double2 v0 = x[j];
             double2 v1 = x[j + quarter], v2 = x[j + 2 * quarter], v3 = x[j + 3 * quarter];
             if (ns > 1) {   // the first stage's twiddles are all 1
-                double2 t1 = __ldg(tw + k * step), t2 = __ldg(tw + 2 * k * step), t3 = __ldg(tw + 3 * k * step);
+                double2 t1 = __ldg(A.tw + k * step), t2 = __ldg(A.tw + 2 * k * step), t3 = __ldg(A.tw + 3 * k * step);
                 if (inverse) {
-                    t1.y = -t1.y;
-                    t2.y = -t2.y;
-                    t3.y = -t3.y;
+                    t1 = conj_of(t1);
+                    t2 = conj_of(t2);
+                    t3 = conj_of(t3);
                 }
                 v1 = cmul(v1, t1);
                 v2 = cmul(v2, t2);
                 v3 = cmul(v3, t3);
             }
             const double2 a0 = cadd(v0, v2), a1 = csub(v0, v2), a2 = cadd(v1, v3), d = csub(v1, v3);
-            // (v1 - v3) times -i (forward) or +i (inverse)
-            const double2 a3 = inverse ? make_double2(-d.y, d.x) : make_double2(d.y, -d.x);
-            const int o = ((j - k) << 2) + k;
-            y[o] = cadd(a0, a2);
-            y[o + ns] = cadd(a1, a3);
-            y[o + 2 * ns] = csub(a0, a2);
-            y[o + 3 * ns] = csub(a1, a3);
+            // (v1 - v3) times -i (forward) or +i (inverse) joins a1
+            const double2 p = make_double2(a1.x - d.y, a1.y + d.x), m = make_double2(a1.x + d.y, a1.y - d.x);
+            o[i][0] = cadd(a0, a2);
+            o[i][2] = csub(a0, a2);
+            o[i][1] = inverse ? p : m;
+            o[i][3] = inverse ? m : p;
         }
         __syncthreads();
-        double2* tmp = x;
-        x = y;
-        y = tmp;
-    }
-    if (ns < n) {   // radix-2 stage, Ns = n/2
-        const int half = n >> 1;
-        const int step = half / ns;
-        for (int j = threadIdx.x; j < half; j += blockDim.x) {
-            const int k = j & (ns - 1);
-            double2 t = __ldg(tw + k * step);
-            if (inverse) t.y = -t.y;
-            const double2 a = x[j];
-            const double2 b = cmul(x[j + half], t);
-            const int o = ((j - k) << 1) + k;
-            y[o] = cadd(a, b);
-            y[o + ns] = csub(a, b);
+#pragma unroll
+        for (int i = 0; i < kMine; ++i) {
+            const int b = tid + i * kNsThreads;
+            if (b >= R * quarter) continue;
+            const int j = b & (quarter - 1), k = j & (ns - 1);
+            double2* y = fft_buf + (b >> lq) * ld + ((j - k) << 2) + k;
+            y[0] = o[i][0];
+            y[ns] = o[i][1];
+            y[2 * ns] = o[i][2];
+            y[3 * ns] = o[i][3];
         }
         __syncthreads();
-        double2* tmp = x;
-        x = y;
-        y = tmp;
     }
-    double2* dst = out + (long long)blockIdx.x * n;
-    if (scale == 1.0)
-        for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = x[i];
-    else
-        for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = cscale(x[i], scale);
-}
-
-// out[c][r] = in[r][c] for a rows x cols complex matrix (32 x 32 tiles)
-__global__ void transpose_kernel(const double2* in, double2* out, int rows, int cols) {
-    __shared__ double2 tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int r = r0 + k, c = c0 + threadIdx.x;
-        if (r < rows && c < cols) tile[k][threadIdx.x] = in[(long long)r * cols + c];
+    if (ns < n) {   // radix-2 stage, Ns = n/2: reads and writes the same two places
+        const int half = n >> 1, lh = lg - 1;
+        for (int b = tid; b < R * half; b += kNsThreads) {
+            const int j = b & (half - 1);
+            double2* x = fft_buf + (b >> lh) * ld;
+            double2 t = __ldg(A.tw + j);
+            if (inverse) t = conj_of(t);
+            const double2 a = x[j], v = cmul(x[j + half], t);
+            x[j] = cadd(a, v);
+            x[j + half] = csub(a, v);
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int c = c0 + k, r = r0 + threadIdx.x;
-        if (r < rows && c < cols) out[(long long)c * rows + r] = tile[threadIdx.x][k];
+    if (STORE == kStoreTransposed) {
+        const int lr = 31 - __clz(R);
+        for (int e = tid; e < count; e += kNsThreads) {
+            const int r = e & (R - 1), c = e >> lr;
+            A.out[which][(long long)c * A.rows + r0 + r] = fft_buf[r * ld + c];
+        }
+    } else {
+        for (int e = tid; e < count; e += kNsThreads) {
+            const int r = e >> lg, c = e & (n - 1);
+            const long long q = ((long long)(r0 + r) << lg) + c;
+            const double2 v = fft_buf[r * ld + c];
+            if (STORE == kStoreRows) {
+                A.out[which][q] = v;
+            } else {
+                if (A.da[which]) A.da[which][q] = v.x;
+                if (A.ta[which]) A.ta[which][q] = (T)v.x;
+                if (A.db[which]) A.db[which][q] = v.y;
+                if (A.tb[which]) A.tb[which][q] = (T)v.y;
+            }
+        }
     }
-}
-
-// Two real fields per complex transform: z = f + i g on the grid (g absent: 0).
-template <typename T>
-__global__ void pack_pair_kernel(const T* f, const T* g, double2* z, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        z[i] = make_double2((double)f[i], g ? (double)g[i] : 0.0);
 }
 
 // Spectra of the two real fields of Z = DFT(f + i g) ([kx][ky], row kx of n1
@@ -154,28 +219,6 @@ __global__ void unpack_pair_kernel(const double2* Z, double2* F, double2* G, int
         const double2 z = Z[q], zm = Z[qm];
         F[q] = make_double2(0.5 * (z.x + zm.x), 0.5 * (z.y - zm.y));
         if (G) G[q] = make_double2(0.5 * (z.y + zm.y), -0.5 * (z.x - zm.x));
-    }
-}
-
-// Z = A + i B in spectral space (B absent: 0), for one inverse transform of two
-// real fields: the real part of the result is a, the imaginary part b
-__global__ void pack_spectra_kernel(const double2* A, const double2* B, double2* Z, long long n) {
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
-        const double2 a = A[q];
-        Z[q] = B ? make_double2(a.x - B[q].y, a.y + B[q].x) : a;
-    }
-}
-
-// real and imaginary parts of z into the FP64 fields da, db and the caller's
-// fields ta, tb (each when given)
-template <typename T>
-__global__ void unpack_grid_kernel(const double2* z, double* da, T* ta, double* db, T* tb, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const double2 v = z[i];
-        if (da) da[i] = v.x;
-        if (ta) ta[i] = (T)v.x;
-        if (db) db[i] = v.y;
-        if (tb) tb[i] = (T)v.y;
     }
 }
 
@@ -207,81 +250,105 @@ __global__ void ns_project_kernel(double2* ux, double2* uy, int n0, int n1, doub
     }
 }
 
-// spectral velocity gradient: g0 = d_x ux, g1 = d_y ux, g2 = d_x uy, g3 = d_y uy
-__global__ void ns_gradient_kernel(const double2* ux, const double2* uy, double2* g0, double2* g1, double2* g2,
-                                   double2* g3, int n0, int n1, double sx, double sy) {
+// Inputs of the three inverse transforms of the velocity (ux, uy) at mode (dx, dy),
+// times scale: ux + i uy, and per component d_x u + i d_y u = (-dy + i dx) u
+// (the gradient entries 0, 1 and 2, 3 of kappa as real and imaginary parts).
+__device__ __forceinline__ void pack_velocity(double2 ux, double2 uy, double dx, double dy, double scale, double2* zu,
+                                              double2* z0, double2* z1) {
+    const double2 a = cscale(ux, scale), b = cscale(uy, scale);
+    *zu = make_double2(a.x - b.y, a.y + b.x);
+    *z0 = make_double2(-dy * a.x - dx * a.y, dx * a.x - dy * a.y);
+    *z1 = make_double2(-dy * b.x - dx * b.y, dx * b.x - dy * b.y);
+}
+
+__global__ void ns_pack_kernel(const double2* ux, const double2* uy, double2* zu, double2* z0, double2* z1, int n0,
+                               int n1, double sx, double sy, double scale) {
     NS_LOOP(q, (long long)n0 * n1) {
         double dx, dy;
         wavenumbers(q, n0, n1, sx, sy, dx, dy);
-        g0[q] = cimul(dx, ux[q]);
-        g1[q] = cimul(dy, ux[q]);
-        g2[q] = cimul(dx, uy[q]);
-        g3[q] = cimul(dy, uy[q]);
+        pack_velocity(ux[q], uy[q], dx, dy, scale, zu + q, z0 + q, z1 + q);
     }
 }
 
-// spectral divergence of the packed stress (xx, xy, yy): (d_x s_xx + d_y s_xy, d_x s_xy + d_y s_yy)
-__global__ void ns_divstress_kernel(const double2* sxx, const double2* sxy, const double2* syy, double2* dx_out,
-                                    double2* dy_out, int n0, int n1, double sx, double sy) {
-    NS_LOOP(q, (long long)n0 * n1) {
-        double dx, dy;
-        wavenumbers(q, n0, n1, sx, sy, dx, dy);
-        dx_out[q] = cadd(cimul(dx, sxx[q]), cimul(dy, sxy[q]));
-        dy_out[q] = cadd(cimul(dx, sxy[q]), cimul(dy, syy[q]));
-    }
-}
-
-// convective term on the grid: (u.grad)u_a = u_x kappa_a,x + u_y kappa_a,y (kappa [4][N] row-major)
-__global__ void ns_convection_kernel(const double* u, const double* kap, double* cx, double* cy, long long N) {
-    NS_LOOP(p, N) {
-        const double ux = u[p], uy = u[N + p];
-        cx[p] = ux * kap[p] + uy * kap[N + p];
-        cy[p] = ux * kap[2 * N + p] + uy * kap[3 * N + p];
-    }
-}
-
-// One step per Fourier mode.  a: u^n, b: u^{n-1}; c, d: the convective term and
-// the stress divergence at levels n (0) and n-1 (1); out: u^{n+1}.
-struct NsModes {
-    const double2 *ax, *ay, *bx, *by;
-    const double2 *c0x, *c0y, *c1x, *c1y;
-    const double2 *d0x, *d0y, *d1x, *d1y;
-    double2 *ox, *oy;
-};
-
-// Per mode, with h = (b1 u^n + b2 u^{n-1})/dt and w = h + E(conv - div sigma):
-// Xi = h + E(nu curl curl u + conv - div sigma), p = i k.Xi / k^2 (Lap p =
+// One step per Fourier mode.  With the explicit terms f = (u.grad)u - div sigma
+// (div sigma up to a gradient: of (xx - yy) and xy alone), h = (b1 u^n + b2 u^{n-1})/dt
+// and w = h + E(f): Xi = h + E(nu curl curl u + f), p = i k.Xi / k^2 (Lap p =
 // -div Xi), (b0/dt + nu k^2) u^{n+1} = -i k p - w.  In Fourier space
 // k.(curl curl u) = k.(k^2 u - k (k.u)) = 0 for every k, so k.Xi = k.w and
 //   u^{n+1} = -(w - k (k.w)/k^2) / (b0/dt + nu k^2),
 // the projection of -w onto divergence-free fields, which the kernel forms
 // directly (the rotational term changes the pressure of the scheme only on a
 // bounded domain).  Mode 0: u^{n+1} = -w dt/b0.
-__global__ void ns_update_kernel(const NsModes M, int n0, int n1, double sx, double sy, double nu, double dt) {
-    const double idt = 1.0 / dt, b0dt = kB0 / dt;
+// Zc, Zs: the forward transforms of the convective term and of the stress
+// (nullptr: none), split by Hermitian symmetry; f1: twice f at level n-1 (nullptr: the
+// empty past, f^{n-1} = f^n); f2 receives twice f^n; u^{n+1} goes over u^{n-1}.
+struct NsModes {
+    const double2 *Zc, *Zs;
+    const double2 *ax, *ay;       // u^n
+    double2 *bx, *by;             // u^{n-1} in, u^{n+1} out
+    const double2 *f1x, *f1y;
+    double2 *f2x, *f2y;
+    double2 *zu, *z0, *z1;        // packed for the inverse transforms
+};
+
+// 2 f at entry q (mode (i, j)) from the two transforms
+__device__ __forceinline__ void explicit_terms(const double2* Zc, const double2* Zs, long long q, long long qm,
+                                               double dx, double dy, double2& fx, double2& fy) {
+    const double2 z = Zc[q], zm = Zc[qm];
+    fx = make_double2(z.x + zm.x, z.y - zm.y);
+    fy = make_double2(z.y + zm.y, zm.x - z.x);
+    if (!Zs) return;
+    const double2 s = Zs[q], sm = Zs[qm];
+    const double2 D = make_double2(s.x + sm.x, s.y - sm.y), S = make_double2(s.y + sm.y, sm.x - s.x);
+    // minus i (dx D + dy S, dx S)
+    fx.x += dx * D.y + dy * S.y;
+    fx.y -= dx * D.x + dy * S.x;
+    fy.x += dx * S.y;
+    fy.y -= dx * S.x;
+}
+
+__device__ __forceinline__ long long mirrored(long long q, int n0, int n1) {
+    const int i = (int)q / n1, j = (int)q - i * n1;
+    return (long long)(i == 0 ? 0 : n0 - i) * n1 + (j == 0 ? 0 : n1 - j);
+}
+
+__global__ void __launch_bounds__(kNsThreads) ns_update_kernel(const NsModes M, int n0, int n1, double sx, double sy,
+                                                               double nu, double b0dt, double b1dt, double b2dt,
+                                                               double inv0, double scale) {
     NS_LOOP(q, (long long)n0 * n1) {
         double dx, dy;
         wavenumbers(q, n0, n1, sx, sy, dx, dy);
+        double2 fx, fy;
+        explicit_terms(M.Zc, M.Zs, q, mirrored(q, n0, n1), dx, dy, fx, fy);
+        // w = h + 2 f^n - f^{n-1}; without a past f^{n-1} = f^n
+        const double2 gx = M.f1x ? M.f1x[q] : fx, gy = M.f1y ? M.f1y[q] : fy;
+        M.f2x[q] = fx;
+        M.f2y[q] = fy;
+        const double2 ax = M.ax[q], ay = M.ay[q], bx = M.bx[q], by = M.by[q];
+        auto w1 = [&](double a, double b, double f, double g) { return fma(-0.5, g, f + fma(b1dt, a, b2dt * b)); };
+        double2 wx = make_double2(w1(ax.x, bx.x, fx.x, gx.x), w1(ax.y, bx.y, fx.y, gx.y));
+        double2 wy = make_double2(w1(ay.x, by.x, fy.x, gy.x), w1(ay.y, by.y, fy.y, gy.y));
         const double k2 = dx * dx + dy * dy;
-        auto wcomp = [&](double2 a, double2 b, double2 c0, double2 c1, double2 d0, double2 d1) {
-            const double2 h = cscale(cadd(cscale(a, kB1), cscale(b, kB2)), idt);
-            return cadd(h, csub(cscale(csub(c0, d0), 2.0), csub(c1, d1)));
-        };
-        double2 wx = wcomp(M.ax[q], M.bx[q], M.c0x[q], M.c1x[q], M.d0x[q], M.d1x[q]);
-        double2 wy = wcomp(M.ay[q], M.by[q], M.c0y[q], M.c1y[q], M.d0y[q], M.d1y[q]);
-        double inv = dt / kB0;
+        double inv = inv0;
         if (k2 > 0.0) {
             // one division gives both 1/k^2 and 1/(b0/dt + nu k^2)
             const double den = b0dt + nu * k2;
-            const double r = 1.0 / (k2 * den);
-            const double2 s = cscale(cadd(cscale(wx, dx), cscale(wy, dy)), den * r);   // (k.w)/k^2
-            wx = csub(wx, cscale(s, dx));
-            wy = csub(wy, cscale(s, dy));
+            const double r = 1.0 / (k2 * den), ik2 = den * r;
+            const double2 s = make_double2((dx * wx.x + dy * wy.x) * ik2, (dx * wx.y + dy * wy.y) * ik2);   // (k.w)/k^2
+            wx = make_double2(fma(-dx, s.x, wx.x), fma(-dx, s.y, wx.y));
+            wy = make_double2(fma(-dy, s.x, wy.x), fma(-dy, s.y, wy.y));
             inv = k2 * r;
         }
-        M.ox[q] = cscale(wx, -inv);
-        M.oy[q] = cscale(wy, -inv);
+        const double2 ux = cscale(wx, -inv), uy = cscale(wy, -inv);
+        M.bx[q] = ux;
+        M.by[q] = uy;
+        pack_velocity(ux, uy, dx, dy, scale, M.zu + q, M.z0 + q, M.z1 + q);
     }
+}
+
+// twice f (no stress) of a level from the transform of its convective term
+__global__ void ns_terms_kernel(const double2* Zc, double2* fx, double2* fy, int n0, int n1) {
+    NS_LOOP(q, (long long)n0 * n1) explicit_terms(Zc, nullptr, q, mirrored(q, n0, n1), 0.0, 0.0, fx[q], fy[q]);
 }
 
 }  // namespace
@@ -297,18 +364,15 @@ struct tfs_ns_ctx {
     int precision = TFS_FP64;
     char* ws = nullptr;
     size_t ws_bytes = 0;
-    // spectral (complex, [kx][ky]): velocity levels, convective term and stress
-    // divergence levels, stress components, gradient components, transposes
-    double2* uh[2][2] = {};       // [level slot][component]
-    double2* ch[2][2] = {};
-    double2* dh[2][2] = {};
-    double2* sh[3] = {};
-    double2* gh[4] = {};
-    double2* tmp[2] = {};
-    // grid fields (FP64): u^n [2][N], kappa^n [4][N], convective term [2][N]
+    // spectral (complex, [kx][ky]): velocity levels and twice the explicit terms
+    // of levels n and n-1 ([level slot][component]); the transforms' inputs and outputs
+    double2* uh[2][2] = {};
+    double2* fh[2][2] = {};
+    double2* za[3] = {};
+    double2* zb[3] = {};
+    // grid fields (FP64): u^n [2][N], kappa^n [4][N]
     double* u = nullptr;
     double* kap = nullptr;
-    double* conv = nullptr;
     double2* tw0 = nullptr;       // exp(-2 pi i t / n0), t < n0; and for n1
     double2* tw1 = nullptr;
     std::vector<double2> tw_host; // both tables, uploaded by tfs_ns_set_state
@@ -325,7 +389,7 @@ size_t ns_up(size_t v) { return (v + kNsAlign - 1) / kNsAlign * kNsAlign; }
 
 size_t ns_bytes(const tfs_ns_ctx* h) {
     const size_t cplx = ns_up(sizeof(double2) * (size_t)h->N), real = ns_up(sizeof(double) * (size_t)h->N);
-    return 21 * cplx + 8 * real + ns_up(sizeof(double2) * (size_t)(h->n0 + h->n1));
+    return 14 * cplx + 6 * real + ns_up(sizeof(double2) * (size_t)(h->n0 + h->n1));
 }
 
 void ns_layout(tfs_ns_ctx* h) {
@@ -335,18 +399,13 @@ void ns_layout(tfs_ns_ctx* h) {
     for (int l = 0; l < 2; ++l)
         for (int a = 0; a < 2; ++a) h->uh[l][a] = take_c();
     for (int l = 0; l < 2; ++l)
-        for (int a = 0; a < 2; ++a) h->ch[l][a] = take_c();
-    for (int l = 0; l < 2; ++l)
-        for (int a = 0; a < 2; ++a) h->dh[l][a] = take_c();
-    for (int c = 0; c < 3; ++c) h->sh[c] = take_c();
-    for (int c = 0; c < 4; ++c) h->gh[c] = take_c();
-    for (int c = 0; c < 2; ++c) h->tmp[c] = take_c();
+        for (int a = 0; a < 2; ++a) h->fh[l][a] = take_c();
+    for (int c = 0; c < 3; ++c) h->za[c] = take_c();
+    for (int c = 0; c < 3; ++c) h->zb[c] = take_c();
     h->u = (double*)p;
     p += 2 * real;
     h->kap = (double*)p;
     p += 4 * real;
-    h->conv = (double*)p;
-    p += 2 * real;
     h->tw0 = (double2*)p;
     h->tw1 = h->tw0 + h->n0;
 }
@@ -356,76 +415,80 @@ unsigned ns_grid(long long n) {
     return (unsigned)(b > 4096 ? 4096 : (b < 1 ? 1 : b));
 }
 
-cudaError_t fft_rows(const tfs_ns_ctx* h, const double2* in, double2* out, int n, int rows, double sign,
-                     double scale, cudaStream_t s) {
-    const int threads = n / 2 < kNsThreads ? (n / 2 > 0 ? n / 2 : 1) : kNsThreads;
-    const double2* tw = n == h->n0 ? h->tw0 : h->tw1;
-    fft_rows_kernel<<<rows, threads, 2 * n * sizeof(double2), s>>>(in, out, n, tw, sign > 0 ? 1 : 0, scale);
+// one pass over the rows of `arrays` arrays: axis 0 rows of n0, axis 1 rows of n1
+template <typename T, int LOAD, int STORE>
+cudaError_t row_pass(const tfs_ns_ctx* h, RowPass<T>& A, int axis, int arrays, bool inverse, cudaStream_t s) {
+    A.n = axis == 0 ? h->n0 : h->n1;
+    A.rows = axis == 0 ? h->n1 : h->n0;
+    A.per_block = kRowElems / A.n < A.rows ? kRowElems / A.n : A.rows;
+    while (A.per_block > 1 && A.rows / A.per_block < kRowBlocks) A.per_block /= 2;
+    A.tw = axis == 0 ? h->tw0 : h->tw1;
+    A.inverse = inverse ? 1 : 0;
+    A.N = h->N;
+    const size_t smem = (size_t)A.per_block * (A.n + 1) * sizeof(double2);
+    fft_pass_kernel<T, LOAD, STORE><<<dim3(A.rows / A.per_block, arrays), kNsThreads, smem, s>>>(A);
     return cudaGetLastError();
 }
 
-cudaError_t transpose(const double2* in, double2* out, int rows, int cols, cudaStream_t s) {
-    transpose_kernel<<<dim3((cols + 31) / 32, (rows + 31) / 32), dim3(32, 8), 0, s>>>(in, out, rows, cols);
-    return cudaGetLastError();
+// Z [kx][ky] = DFT of what the first pass loads
+template <typename T, int LOAD>
+cudaError_t forward(const tfs_ns_ctx* h, RowPass<T> A, double2* Z, cudaStream_t s) {
+    A.out[0] = Z;
+    return row_pass<T, LOAD, kStoreTransposed>(h, A, 0, 1, false, s);
+}
+template <typename T>
+cudaError_t forward_second(const tfs_ns_ctx* h, double2* Z0, double2* Z1, cudaStream_t s) {
+    RowPass<T> A{};
+    A.in[0] = A.out[0] = Z0;
+    A.in[1] = A.out[1] = Z1;
+    return row_pass<T, kLoadComplex, kStoreRows>(h, A, 1, Z1 ? 2 : 1, false, s);
 }
 
-// spectra [kx][ky] of two real grid fields [y][x] (g absent: G not formed),
-// by one complex transform of f + i g
+// spectra of two real fields by one transform of f + i g
 template <typename T>
 cudaError_t fft2_pair(tfs_ns_ctx* h, const T* f, const T* g, double2* F, double2* G, cudaStream_t s) {
-    pack_pair_kernel<T><<<ns_grid(h->N), kNsThreads, 0, s>>>(f, g, h->tmp[0], h->N);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = fft_rows(h, h->tmp[0], h->tmp[0], h->n0, h->n1, -1.0, 1.0, s);
-    if (e == cudaSuccess) e = transpose(h->tmp[0], h->tmp[1], h->n1, h->n0, s);
-    if (e == cudaSuccess) e = fft_rows(h, h->tmp[1], h->tmp[1], h->n1, h->n0, -1.0, 1.0, s);
+    RowPass<T> A{};
+    A.f = f;
+    A.g = g;
+    cudaError_t e = forward<T, kLoadPair>(h, A, h->za[0], s);
+    if (e == cudaSuccess) e = forward_second<T>(h, h->za[0], nullptr, s);
     if (e == cudaSuccess) {
-        unpack_pair_kernel<<<ns_grid(h->N), kNsThreads, 0, s>>>(h->tmp[1], F, G, h->n0, h->n1);
+        unpack_pair_kernel<<<ns_grid(h->N), kNsThreads, 0, s>>>(h->za[0], F, G, h->n0, h->n1);
         e = cudaGetLastError();
     }
     return e;
 }
 
-// real grid fields [y][x] of the spectra A and B ([kx][ky], both Hermitian; B
-// may be absent), by one inverse transform of A + i B: a into da and/or ta, b
-// into db and/or tb
-template <typename T>
-cudaError_t ifft2_pair(tfs_ns_ctx* h, const double2* A, const double2* B, double* da, T* ta, double* db, T* tb,
-                       cudaStream_t s) {
-    pack_spectra_kernel<<<ns_grid(h->N), kNsThreads, 0, s>>>(A, B, h->tmp[0], h->N);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = fft_rows(h, h->tmp[0], h->tmp[0], h->n1, h->n0, 1.0, 1.0, s);
-    if (e == cudaSuccess) e = transpose(h->tmp[0], h->tmp[1], h->n0, h->n1, s);
-    if (e == cudaSuccess) e = fft_rows(h, h->tmp[1], h->tmp[1], h->n0, h->n1, 1.0, 1.0 / (double)h->N, s);
-    if (e == cudaSuccess) {
-        unpack_grid_kernel<T><<<ns_grid(h->N), kNsThreads, 0, s>>>(h->tmp[1], da, ta, db, tb, h->N);
-        e = cudaGetLastError();
-    }
-    return e;
-}
-
-// grid velocity and gradient of the spectral level (ux, uy) into the FP64
+// grid velocity and gradient of the packed spectra in za (zu, z0, z1): into the FP64
 // fields u, kap and, when given, the caller's fields uo [2][N], ko [4][N]
 template <typename T>
-cudaError_t grid_fields(tfs_ns_ctx* h, double2* ux, double2* uy, double* u, double* kap, T* uo, T* ko,
-                        cudaStream_t s) {
+cudaError_t grid_fields(tfs_ns_ctx* h, T* uo, T* ko, cudaStream_t s) {
     const long long N = h->N;
-    cudaError_t e = ifft2_pair<T>(h, ux, uy, u, uo, u + N, uo ? uo + N : nullptr, s);
+    RowPass<T> A{};
+    for (int c = 0; c < 3; ++c) {
+        A.in[c] = h->za[c];
+        A.out[c] = h->zb[c];
+    }
+    cudaError_t e = row_pass<T, kLoadComplex, kStoreTransposed>(h, A, 1, 3, true, s);
     if (e != cudaSuccess) return e;
-    ns_gradient_kernel<<<ns_grid(N), kNsThreads, 0, s>>>(ux, uy, h->gh[0], h->gh[1], h->gh[2], h->gh[3], h->n0, h->n1,
-                                                         h->sx, h->sy);
-    e = cudaGetLastError();
-    for (int c = 0; c < 4 && e == cudaSuccess; c += 2)
-        e = ifft2_pair<T>(h, h->gh[c], h->gh[c + 1], kap + c * N, ko ? ko + c * N : nullptr, kap + (c + 1) * N,
-                          ko ? ko + (c + 1) * N : nullptr, s);
-    return e;
+    for (int c = 0; c < 3; ++c) {
+        double* d = c == 0 ? h->u : h->kap + (c == 1 ? 0 : 2) * N;
+        T* t = c == 0 ? uo : (ko ? ko + (c == 1 ? 0 : 2) * N : nullptr);
+        A.in[c] = h->zb[c];
+        A.da[c] = d;
+        A.db[c] = d + N;
+        A.ta[c] = t;
+        A.tb[c] = t ? t + N : nullptr;
+    }
+    return row_pass<T, kLoadComplex, kStoreFields>(h, A, 0, 3, true, s);
 }
 
-// spectral convective term (u.grad)u of grid fields u, kap into (cx, cy)
-cudaError_t convection(tfs_ns_ctx* h, const double* u, const double* kap, double2* cx, double2* cy, cudaStream_t s) {
-    ns_convection_kernel<<<ns_grid(h->N), kNsThreads, 0, s>>>(u, kap, h->conv, h->conv + h->N, h->N);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = fft2_pair<double>(h, h->conv, h->conv + h->N, cx, cy, s);
-    return e;
+template <typename T>
+cudaError_t fields_of_level(tfs_ns_ctx* h, const double2* ux, const double2* uy, cudaStream_t s) {
+    ns_pack_kernel<<<ns_grid(h->N), kNsThreads, 0, s>>>(ux, uy, h->za[0], h->za[1], h->za[2], h->n0, h->n1, h->sx,
+                                                        h->sy, 1.0 / (double)h->N);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? grid_fields<T>(h, nullptr, nullptr, s) : e;
 }
 
 template <typename T>
@@ -446,15 +509,21 @@ int ns_set_state(tfs_ns_ctx* h, const T* u0, const T* uprev, cudaStream_t s) {
             ns_project_kernel<<<ns_grid(N), kNsThreads, 0, s>>>(h->uh[o][0], h->uh[o][1], h->n0, h->n1, h->sx, h->sy);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = grid_fields<T>(h, h->uh[o][0], h->uh[o][1], h->u, h->kap, nullptr, nullptr, s);
-        if (e == cudaSuccess) e = convection(h, h->u, h->kap, h->ch[o][0], h->ch[o][1], s);
-        for (int a = 0; a < 2 && e == cudaSuccess; ++a)
-            e = cudaMemsetAsync(h->dh[o][a], 0, sizeof(double2) * (size_t)N, s);
+        if (e == cudaSuccess) e = fields_of_level<T>(h, h->uh[o][0], h->uh[o][1], s);
+        RowPass<T> A{};
+        A.u = h->u;
+        A.kap = h->kap;
+        if (e == cudaSuccess) e = forward<T, kLoadConvection>(h, A, h->za[0], s);
+        if (e == cudaSuccess) e = forward_second<T>(h, h->za[0], nullptr, s);
+        if (e == cudaSuccess) {
+            ns_terms_kernel<<<ns_grid(N), kNsThreads, 0, s>>>(h->za[0], h->fh[o][0], h->fh[o][1], h->n0, h->n1);
+            e = cudaGetLastError();
+        }
     } else if (e == cudaSuccess) {
         for (int a = 0; a < 2 && e == cudaSuccess; ++a)
             e = cudaMemcpyAsync(h->uh[o][a], h->uh[c][a], sizeof(double2) * (size_t)N, cudaMemcpyDeviceToDevice, s);
     }
-    if (e == cudaSuccess) e = grid_fields<T>(h, h->uh[c][0], h->uh[c][1], h->u, h->kap, nullptr, nullptr, s);
+    if (e == cudaSuccess) e = fields_of_level<T>(h, h->uh[c][0], h->uh[c][1], s);
     if (e != cudaSuccess) return TFS_ERR_CUDA;
     h->have_prev_terms = uprev != nullptr;
     h->state_set = true;
@@ -464,33 +533,25 @@ int ns_set_state(tfs_ns_ctx* h, const T* u0, const T* uprev, cudaStream_t s) {
 
 template <typename T>
 int ns_step(tfs_ns_ctx* h, const T* sigma, T* u_out, T* kap_out, cudaStream_t s) {
-    const long long N = h->N;
     const int c = h->cur, o = 1 - c;
-    // explicit terms of level n: convection from the stored grid fields, stress divergence
-    cudaError_t e = convection(h, h->u, h->kap, h->ch[c][0], h->ch[c][1], s);
-    if (e == cudaSuccess && sigma) {
-        e = fft2_pair<T>(h, sigma, sigma + N, h->sh[0], h->sh[1], s);
-        if (e == cudaSuccess) e = fft2_pair<T>(h, sigma + 2 * N, (const T*)nullptr, h->sh[2], nullptr, s);
-        if (e == cudaSuccess) {
-            ns_divstress_kernel<<<ns_grid(N), kNsThreads, 0, s>>>(h->sh[0], h->sh[1], h->sh[2], h->dh[c][0],
-                                                                  h->dh[c][1], h->n0, h->n1, h->sx, h->sy);
-            e = cudaGetLastError();
-        }
-    } else {
-        for (int a = 0; a < 2 && e == cudaSuccess; ++a)
-            e = cudaMemsetAsync(h->dh[c][a], 0, sizeof(double2) * (size_t)N, s);
-    }
+    // transforms of the convective term (from the stored grid fields) and of the stress
+    RowPass<T> A{};
+    A.u = h->u;
+    A.kap = h->kap;
+    A.f = sigma;
+    cudaError_t e = forward<T, kLoadConvection>(h, A, h->zb[0], s);
+    if (e == cudaSuccess && sigma) e = forward<T, kLoadStress>(h, A, h->zb[1], s);
+    if (e == cudaSuccess) e = forward_second<T>(h, h->zb[0], sigma ? h->zb[1] : nullptr, s);
     if (e != cudaSuccess) return TFS_ERR_CUDA;
-    // level n-1's terms (the empty past: level n's)
-    const int pc = h->have_prev_terms ? o : c;
-    NsModes M{h->uh[c][0], h->uh[c][1], h->uh[o][0], h->uh[o][1],
-              h->ch[c][0], h->ch[c][1], h->ch[pc][0], h->ch[pc][1],
-              h->dh[c][0], h->dh[c][1], h->dh[pc][0], h->dh[pc][1],
-              h->uh[o][0], h->uh[o][1]};
     // u^{n+1} is written over u^{n-1}: each mode reads its own entries before writing them
-    ns_update_kernel<<<ns_grid(N), kNsThreads, 0, s>>>(M, h->n0, h->n1, h->sx, h->sy, h->nu, h->dt);
+    const bool past = h->have_prev_terms;
+    const NsModes M{h->zb[0], sigma ? h->zb[1] : nullptr, h->uh[c][0], h->uh[c][1], h->uh[o][0], h->uh[o][1],
+                    past ? h->fh[o][0] : nullptr, past ? h->fh[o][1] : nullptr, h->fh[c][0], h->fh[c][1],
+                    h->za[0], h->za[1], h->za[2]};
+    ns_update_kernel<<<ns_grid(h->N), kNsThreads, 0, s>>>(M, h->n0, h->n1, h->sx, h->sy, h->nu, kB0 / h->dt,
+                                                          kB1 / h->dt, kB2 / h->dt, h->dt / kB0, 1.0 / (double)h->N);
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = grid_fields<T>(h, h->uh[o][0], h->uh[o][1], h->u, h->kap, u_out, kap_out, s);
+    if (e == cudaSuccess) e = grid_fields<T>(h, u_out, kap_out, s);
     if (e != cudaSuccess) return TFS_ERR_CUDA;
     h->cur = o;
     h->have_prev_terms = true;

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kThreads) paper_adjoint_kernel(const PaperAdjA
             const long long q = (long long)c * N + p;
             A.s1_out[q] = A.s0[q] - kB1 * (double)lam[c];
             A.s0_out[q] = -kB2 * (double)lam[c];
-            if (A.lamR_out) A.lamR_out[q] = (double)lam[c];
+            if (A.lamR_out) A.lamR_out[q] = (T)lam[c];
         }
         // parameter derivatives (the stress form's with sigma^{n+1} -> Psi^{n+1})
         R S3[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};

@@ -33,7 +33,7 @@ struct PaperAdjArgs {
     const double* t0;
     double* t1_out;
     double* t0_out;
-    double* lamR_out;
+    T* lamR_out;
     double* partials;
     unsigned* flags;
     long long N;

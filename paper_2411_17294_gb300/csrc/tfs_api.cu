@@ -1394,7 +1394,7 @@ cudaError_t paper_adjoint_step(const tfs_ctx* h, const AdjLayout& L, int cur, in
         a.t0 = L.t[2 * cur + 1];
         a.t1_out = L.t[2 * nxt];
         a.t0_out = L.t[2 * nxt + 1];
-        a.lamR_out = L.lamR;
+        a.lamR_out = (T*)L.lamR;
     }
     a.partials = L.partials;
     a.flags = h->flags;
@@ -1422,10 +1422,9 @@ cudaError_t paper_adjoint_step(const tfs_ctx* h, const AdjLayout& L, int cur, in
     ad.dt = h->dt;
     ad.eps = h->eps;
     for (int i = 0; i < 3; ++i) ad.inv_h[i] = (double)h->n[i] / h->L[i];
-    ad.lamR = L.lamR;
     ad.s1_out = L.t[2 * nxt];
     ad.s0_out = L.t[2 * nxt + 1];
-    return launch_adjoint_transport(ad, u, sizeof(T) == 8, make_cfg(h), s);
+    return launch_adjoint_transport(ad, L.lamR, u, sizeof(T) == 8, make_cfg(h), s);
 }
 
 // Psi0^{n+1} of steps 0 .. steps-1 (with the SDIRK2 start: Psi0 at its two
@@ -1736,7 +1735,7 @@ static int backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* ch
                 h->last_relres = rr;
             }
             if (e == cudaSuccess) e = launch_adjoint_f64(a, cfg, s);
-            if (e == cudaSuccess && h->explicit_transport()) e = launch_adjoint_transport(a, u, true, cfg, s);
+            if (e == cudaSuccess && h->explicit_transport()) e = launch_adjoint_transport(a, a.lamR, u, true, cfg, s);
         } else {
             AdjArgs<float> a{};
             a.kap_n = (const float*)grad_u;
@@ -1751,7 +1750,7 @@ static int backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* ch
             a.s0 = L.s[2 * cur + 1];
             a.s1_out = L.s[2 * nxt];
             a.s0_out = L.s[2 * nxt + 1];
-            a.lamR = L.lamR;
+            a.lamR = (float*)L.lamR;
             a.g_sigma0 = dJ_dsigma0;
             a.g_kap = dJ_dgrad_u;
             a.partials = L.partials;
@@ -1791,10 +1790,9 @@ static int backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* ch
                 ad.dt = a.dt;
                 ad.eps = a.eps;
                 for (int i = 0; i < 3; ++i) ad.inv_h[i] = a.inv_h[i];
-                ad.lamR = a.lamR;
                 ad.s1_out = a.s1_out;
                 ad.s0_out = a.s0_out;
-                e = launch_adjoint_transport(ad, u, false, cfg, s);
+                e = launch_adjoint_transport(ad, a.lamR, u, false, cfg, s);
             }
         }
         if (e != cudaSuccess) return TFS_ERR_CUDA;

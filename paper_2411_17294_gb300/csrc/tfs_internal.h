@@ -262,7 +262,7 @@ struct AdjArgs {
     const double* s0;      // [nc][N]
     double* s1_out;        // adjoint of sigma^n       (next step's s1)
     double* s0_out;        // adjoint of sigma^{n-1}   (next step's s0)
-    double* lamR;          // [nc][N] scratch: adjoint of the right-hand side (for transport)
+    T* lamR;               // [nc][N] scratch: adjoint of the right-hand side (for transport)
     // adjoint mode ring: ell_prev = lamQ of the previous adjoint step, ell_prev2 the one before
     const T* ell_prev;     // [m][nc][N]
     T* ell_prev2;          // [m][nc][N] read, then overwritten with this step's lamQ
@@ -282,7 +282,8 @@ struct AdjArgs {
 
 cudaError_t launch_adjoint_f64(const AdjArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s);
 cudaError_t launch_adjoint_f32(const AdjArgs<float>& a, const LaunchCfg& cfg, cudaStream_t s);
-cudaError_t launch_adjoint_transport(const AdjArgs<double>& a, const void* u, bool u_is_double,
+// a.lamR is not used: lamR and u are of the storage type
+cudaError_t launch_adjoint_transport(const AdjArgs<double>& a, const void* lamR, const void* u, bool is_double,
                                      const LaunchCfg& cfg, cudaStream_t s);
 cudaError_t launch_reduce_partials(const double* partials, int count, double* out2, cudaStream_t s);
 

@@ -1,4 +1,5 @@
-// Adjoint (reverse-mode derivative) of one forward stress step.
+// Adjoint (reverse-mode derivative) of one forward stress step: FP32 storage
+// (FP64: tfs_adjoint64.cu), and the transposed transport stencil of both.
 //
 // The forward step maps (sigma^n, sigma^{n-1}, modes^n, modes^{n-1}) to
 // (sigma^{n+1}, sigma^n, modes^{n+1}, modes^n).  Its push-forward
@@ -155,10 +156,10 @@ struct AdjShape {
 };
 
 // Resident blocks asked of the register allocator: the most that compile
-// without spills (2D: 6; 3D: 5 in FP32, 4 in FP64).
+// without spills.
 template <typename T, int DIM>
 constexpr int adj_min_blocks() {
-    return DIM == 2 ? 6 : (sizeof(T) == 4 ? 5 : 4);
+    return DIM == 2 ? 6 : 5;
 }
 
 // One tile.  `after_pass1` runs on all threads right after the barrier that
@@ -170,7 +171,7 @@ __device__ __forceinline__ void adj_tile(const AdjArgs<T>& A, const AdjStageMap&
     constexpr int NC = Packed<DIM>::NC;
     constexpr int W = AdjShape<DIM>::W;
     constexpr int CPW = AdjShape<DIM>::CPW;
-    constexpr bool F32 = sizeof(T) == 4;
+    static_assert(sizeof(T) == 4, "FP64 storage: tfs_adjoint64.cu");
     T* tb = reinterpret_cast<T*>(buf);
     const double* db = reinterpret_cast<const double*>(buf + (size_t)S.tplanes * kTileA * sizeof(T));
     const int lane = threadIdx.x;
@@ -184,43 +185,25 @@ __device__ __forceinline__ void adj_tile(const AdjArgs<T>& A, const AdjStageMap&
     if (!classic) {
         const T* e1 = tb + (S.e1 + w) * kTileA + lane;
         T* e2 = tb + (S.e2 + w) * kTileA + lane;
-        if constexpr (F32) {
-            float ss[CPW], comp[CPW];
+        float ss[CPW], comp[CPW];
 #pragma unroll
-            for (int cc = 0; cc < CPW; ++cc) ss[cc] = comp[cc] = 0.0f;
+        for (int cc = 0; cc < CPW; ++cc) ss[cc] = comp[cc] = 0.0f;
 #pragma unroll 4
-            for (int j = 0; j < m; ++j) {
-                const float rh = A.mcf.rho[j];
+        for (int j = 0; j < m; ++j) {
+            const float rh = A.mcf.rho[j];
 #pragma unroll
-                for (int cc = 0; cc < CPW; ++cc) {
-                    const int o = (j * NC + cc * W) * kTileA;
-                    const float z = A.first ? 0.0f : __fmaf_rn(0.5f, e2[o], -2.0f * e1[o]);
-                    e2[o] = z;
-                    const float yv = __fmaf_rn(rh, z, -comp[cc]);
-                    const float t = __fadd_rn(ss[cc], yv);
-                    comp[cc] = __fsub_rn(__fsub_rn(t, ss[cc]), yv);
-                    ss[cc] = t;
-                }
+            for (int cc = 0; cc < CPW; ++cc) {
+                const int o = (j * NC + cc * W) * kTileA;
+                const float z = A.first ? 0.0f : __fmaf_rn(0.5f, e2[o], -2.0f * e1[o]);
+                e2[o] = z;
+                const float yv = __fmaf_rn(rh, z, -comp[cc]);
+                const float t = __fadd_rn(ss[cc], yv);
+                comp[cc] = __fsub_rn(__fsub_rn(t, ss[cc]), yv);
+                ss[cc] = t;
             }
-#pragma unroll
-            for (int cc = 0; cc < CPW; ++cc) sS[(w + cc * W) * kTileA + lane] = (double)ss[cc] - (double)comp[cc];
-        } else {
-            double ss[CPW];
-#pragma unroll
-            for (int cc = 0; cc < CPW; ++cc) ss[cc] = 0.0;
-#pragma unroll 2
-            for (int j = 0; j < m; ++j) {
-#pragma unroll
-                for (int cc = 0; cc < CPW; ++cc) {
-                    const int o = (j * NC + cc * W) * kTileA;
-                    const double z = A.first ? 0.0 : kB1 * (double)e1[o] + kB2 * (double)e2[o];
-                    e2[o] = (T)z;
-                    ss[cc] = fma(A.mc.rho[j], z, ss[cc]);
-                }
-            }
-#pragma unroll
-            for (int cc = 0; cc < CPW; ++cc) sS[(w + cc * W) * kTileA + lane] = ss[cc];
         }
+#pragma unroll
+        for (int cc = 0; cc < CPW; ++cc) sS[(w + cc * W) * kTileA + lane] = (double)ss[cc] - (double)comp[cc];
     } else {
 #pragma unroll
         for (int cc = 0; cc < CPW; ++cc) sS[(w + cc * W) * kTileA + lane] = 0.0;
@@ -228,11 +211,10 @@ __device__ __forceinline__ void adj_tile(const AdjArgs<T>& A, const AdjStageMap&
     __syncthreads();
     after_pass1();
 
-    // ---- point system and parameter derivatives by warp 0.  FP64 storage:
-    //      FP64 throughout.  FP32 storage: the per-point arithmetic in FP32 (FP32
+    // ---- point system and parameter derivatives by warp 0: the per-point arithmetic in FP32 (FP32
     //      LU of M^T with partial pivoting), accumulations into the FP64 fields.
     if (w == 0) {
-        using R = typename std::conditional<F32, float, double>::type;
+        using R = float;
         R K[3][3];
 #pragma unroll
         for (int a = 0; a < DIM; ++a)
@@ -246,34 +228,24 @@ __device__ __forceinline__ void adj_tile(const AdjArgs<T>& A, const AdjStageMap&
             lam[r] = (R)(db[(S.s1 + r) * kTileA + lane] + sS[r * kTileA + lane]);
         }
         bool ok;
-        if constexpr (F32) {
-            LU32<NC> F;
-            static_for<0, NC>([&](auto rr) {
-                constexpr int r = decltype(rr)::value;
-                static_for<0, NC>([&](auto kk) {
-                    constexpr int k = decltype(kk)::value;
-                    // transpose: entry (r, k) of M^T is entry (k, r) of M
-                    constexpr int ro = Packed<DIM>::I(k), so = Packed<DIM>::J(k);
-                    constexpr int i = Packed<DIM>::I(r), j = Packed<DIM>::J(r);
-                    float v = 0.0f;
-                    if (so == j) v += K[ro][i];
-                    if (i != j && so == i) v += K[ro][j];
-                    if (ro == i) v += K[so][j];
-                    if (i != j && ro == j) v += K[so][i];
-                    F.a[r][k] = (r == k) ? __fmaf_rn(-(float)A.dt, v, (float)A.a) : -(float)A.dt * v;
-                });
+        LU32<NC> F;
+        static_for<0, NC>([&](auto rr) {
+            constexpr int r = decltype(rr)::value;
+            static_for<0, NC>([&](auto kk) {
+                constexpr int k = decltype(kk)::value;
+                // transpose: entry (r, k) of M^T is entry (k, r) of M
+                constexpr int ro = Packed<DIM>::I(k), so = Packed<DIM>::J(k);
+                constexpr int i = Packed<DIM>::I(r), j = Packed<DIM>::J(r);
+                float v = 0.0f;
+                if (so == j) v += K[ro][i];
+                if (i != j && so == i) v += K[ro][j];
+                if (ro == i) v += K[so][j];
+                if (i != j && ro == j) v += K[so][i];
+                F.a[r][k] = (r == k) ? __fmaf_rn(-(float)A.dt, v, (float)A.a) : -(float)A.dt * v;
             });
-            ok = lu32_factor<NC>(F, 1e-30f);
-            lu32_solve<NC>(F, lam);
-        } else {
-            double M[NC][NC], Mt[NC][NC];
-            assemble_M<DIM>(K, A.a, A.dt, M);
-#pragma unroll
-            for (int r = 0; r < NC; ++r)
-#pragma unroll
-                for (int k = 0; k < NC; ++k) Mt[r][k] = M[k][r];
-            ok = gauss_pp<NC>(Mt, lam, 1e-300);
-        }
+        });
+        ok = lu32_factor<NC>(F, 1e-30f);
+        lu32_solve<NC>(F, lam);
         // lam now holds lamR
         R gK[3][3];
 #pragma unroll
@@ -345,28 +317,16 @@ __device__ __forceinline__ void adj_tile(const AdjArgs<T>& A, const AdjStageMap&
         const T* zv = tb + (S.e2 + w) * kTileA + lane;
         T* out = A.ell_prev2 + mode_index(p, w, m * NC);   // tile-major ring, row j NC + c
         constexpr long long stride = (long long)NC * kTileA;
-        if constexpr (F32) {
-            float l[CPW];
+        float l[CPW];
 #pragma unroll
-            for (int cc = 0; cc < CPW; ++cc) l[cc] = (float)sL[(w + cc * W) * kTileA + lane];
+        for (int cc = 0; cc < CPW; ++cc) l[cc] = (float)sL[(w + cc * W) * kTileA + lane];
 #pragma unroll 4
-            for (int j = 0; j < m; ++j) {
-                const float ej = A.mcf.eta_hi[j], cjf = A.mcf.c[j];
+        for (int j = 0; j < m; ++j) {
+            const float ej = A.mcf.eta_hi[j], cjf = A.mcf.c[j];
 #pragma unroll
-                for (int cc = 0; cc < CPW; ++cc)
-                    __stcs(out + j * stride + (long long)cc * W * kTileA,
-                           __fmaf_rn(-ej, l[cc], -cjf * zv[(j * NC + cc * W) * kTileA]));
-            }
-        } else {
-            double l[CPW];
-#pragma unroll
-            for (int cc = 0; cc < CPW; ++cc) l[cc] = sL[(w + cc * W) * kTileA + lane];
-#pragma unroll 2
-            for (int j = 0; j < m; ++j)
-#pragma unroll
-                for (int cc = 0; cc < CPW; ++cc)
-                    __stcs(out + j * stride + (long long)cc * W * kTileA,
-                           (T)fma(-A.mc.eta[j], l[cc], -A.mc.c[j] * (double)zv[(j * NC + cc * W) * kTileA]));
+            for (int cc = 0; cc < CPW; ++cc)
+                __stcs(out + j * stride + (long long)cc * W * kTileA,
+                       __fmaf_rn(-ej, l[cc], -cjf * zv[(j * NC + cc * W) * kTileA]));
         }
     }
 }
@@ -578,10 +538,6 @@ cudaError_t launch_adj(const AdjArgs<T>& a, const LaunchCfg& cfg, cudaStream_t s
 }
 
 }  // namespace
-
-cudaError_t launch_adjoint_f64(const AdjArgs<double>& a, const LaunchCfg& cfg, cudaStream_t s) {
-    return cfg.dim == 2 ? launch_adj<double, 2>(a, cfg, s) : launch_adj<double, 3>(a, cfg, s);
-}
 
 cudaError_t launch_adjoint_f32(const AdjArgs<float>& a, const LaunchCfg& cfg, cudaStream_t s) {
     return cfg.dim == 2 ? launch_adj<float, 2>(a, cfg, s) : launch_adj<float, 3>(a, cfg, s);

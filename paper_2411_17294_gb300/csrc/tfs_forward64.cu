@@ -36,11 +36,11 @@
 
 #include "tfs_device.cuh"
 #include "tfs_internal.h"
+#include "tfs_solve64.cuh"
 
 namespace tfs {
 namespace {
 
-constexpr int kT64 = 32;     // points per tile
 constexpr int kAhead = 8;    // modes whose two levels a thread loads before using them
 
 // where the transport term comes from
@@ -70,12 +70,6 @@ struct Step64 {
     float inv_h[3];
     float a;
 };
-
-// Tests that keep off the FP64 pipe.
-__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
-__device__ __forceinline__ bool zero64(double v) {
-    return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0;
-}
 
 // v >= 0 (-0 included)
 __device__ __forceinline__ bool not_negative(double v) { return __double2hiint(v) >= 0 || zero64(v); }
@@ -161,63 +155,6 @@ __device__ __forceinline__ double stencil_term(const FwdArgs<double>& A, int ste
         }
     }
     return acc;
-}
-
-// ---- FP32 images of FP64 numbers by integer operations (a conversion costs what
-// an FP64 operation does).  A vector is scaled by the power of two that brings
-// its largest component to [1, 2); smaller components lose the bits below that
-// of the float format, which the refinement recovers.
-__device__ __forceinline__ int biased_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
-
-__device__ __forceinline__ float scaled_float(double v, int emax) {
-    const int hi = __double2hiint(v), lo = __double2loint(v);
-    const int be = (hi >> 20) & 0x7ff, e = be - emax + 127;
-    const unsigned bits = ((unsigned)hi & 0x80000000u) | ((unsigned)e << 23) | (((unsigned)hi & 0xfffffu) << 3) |
-                          ((unsigned)lo >> 29);
-    return be > 0 && e > 0 ? __uint_as_float(bits) : 0.0f;
-}
-
-// f 2^(emax - 1023), exactly, for a finite f whose scaled exponent is in range (0 below it).
-__device__ __forceinline__ double unscaled_double(float f, int emax) {
-    const unsigned b = __float_as_uint(f);
-    const int e = (int)((b >> 23) & 0xffu) - 127 + emax;
-    const int hi = (int)((b & 0x80000000u) | ((unsigned)e << 20) | ((b & 0x7fffffu) >> 3));
-    return ((b >> 23) & 0xffu) != 0u && e > 0 ? __hiloint2double(hi, (int)(b << 29)) : 0.0;
-}
-
-// Barrier of the first N threads of a block.
-template <int N>
-__device__ __forceinline__ void named_sync() {
-    asm volatile("bar.sync 1, %0;\n" ::"n"(N) : "memory");
-}
-
-// Packed component of the symmetric entry (a, b).
-template <int DIM>
-struct PackedIndex {
-    __host__ __device__ static constexpr int at(int a, int b) {
-        return a == b ? (DIM == 2 ? 2 * a : a) : (DIM == 2 ? 1 : 6 - a - b);
-    }
-};
-
-// The point system by FP64 Gaussian elimination (K scaled as in the kernel):
-// component c of M^-1 R.  Returns false when a pivot vanishes.
-template <int DIM>
-__device__ __noinline__ bool solve_by_elimination(const double* sK, const double* sR, double a, int c, double* out) {
-    constexpr int NC = Packed<DIM>::NC;
-    double K[3][3], x[NC], M[NC][NC];
-#pragma unroll
-    for (int i = 0; i < DIM; ++i)
-#pragma unroll
-        for (int j = 0; j < DIM; ++j) K[i][j] = sK[(i * DIM + j) * kT64];
-#pragma unroll
-    for (int r = 0; r < NC; ++r) x[r] = sR[r * kT64];
-    assemble_M<DIM>(K, a, 1.0, M);
-    const bool ok = gauss_pp<NC>(M, x, 1e-300);
-    *out = x[0];
-#pragma unroll
-    for (int r = 1; r < NC; ++r)
-        if (c == r) *out = x[r];
-    return ok;
 }
 
 // One tile of 32 points per block; warp (c, g) takes component c and the modes
@@ -344,85 +281,8 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
     }
     __syncthreads();
     if (grp == 0) {
-        // ---- FP32 factors of the 32 matrices, one each per lane, in every warp
-        LU32<NC> F;
-        static_for<0, NC>([&](auto rr) {
-            constexpr int ro = decltype(rr)::value;
-            static_for<0, NC>([&](auto kk) {
-                constexpr int k = decltype(kk)::value;
-                constexpr int i1 = Packed<DIM>::I(ro), j1 = Packed<DIM>::J(ro);
-                constexpr int i = Packed<DIM>::I(k), j = Packed<DIM>::J(k);
-                const float* kf = sKf + lane;
-                float v = ro == k ? B.a : 0.0f;
-                if (j1 == j) v -= kf[(i1 * DIM + i) * kT64];
-                if (i != j && j1 == i) v -= kf[(i1 * DIM + j) * kT64];
-                if (i1 == i) v -= kf[(j1 * DIM + j) * kT64];
-                if (i != j && i1 == j) v -= kf[(j1 * DIM + i) * kT64];
-                F.a[ro][k] = v;
-            });
-        });
-        bool good = row_dominant<NC>(F) ? lu32_factor_nopivot<NC>(F, 1e-30f) : lu32_factor<NC>(F, 1e-30f);
-        // ---- x = y0 + y1 + y2 ...: each y the FP32 solution for the residual so far.  With
-        //      contraction q per pass the error after y2 is |y2| q: q < 2^-18 leaves it below
-        //      the last bit, and then |y2| is below 2^-36 |x|; otherwise further passes
-        int e0 = 0;
-        constexpr int kMaxPass = 8;
-        bool done = false;
-        for (int pass = 0; pass < kMaxPass; ++pass) {
-            const double* rb = pass == 0 ? sR : sR + (1 + (pass & 1)) * NC * kT64;
-            double rv[NC];
-            int emax = 0;
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                rv[k] = rb[k * kT64 + lane];
-                emax = max(emax, biased_exp(rv[k]));
-            }
-            // a residual of zeros (or below the range of a scaled float) is solved
-            bool zero = true;
-            float y[NC];
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                zero = zero && zero64(rv[k]);
-                y[k] = scaled_float(rv[k], emax);
-            }
-            if (pass == 0) good = good && emax < 0x7ff && (emax > 200 || zero);
-            lu32_solve<NC>(F, y);
-            unsigned ymax = 0u;
-#pragma unroll
-            for (int k = 0; k < NC; ++k) ymax = max(ymax, __float_as_uint(y[k]) & 0x7fffffffu);
-            const int ey = (int)(ymax >> 23) + emax;       // exponent of the correction (biased by 127 + 1023)
-            if (pass == 0) {
-                good = good && ymax < 0x7f800000u && ey - 127 < 0x7ff;
-                e0 = ey;
-            }
-            const bool small = ymax == 0u || ey <= e0 - 36;
-            static_for<0, NC>([&](auto kk) {
-                constexpr int k = decltype(kk)::value;
-                // a point's passes are its own, whatever the other points of its tile still need
-                if (c == k && !done) x += unscaled_double(y[k], emax);
-            });
-            done = done || zero || (pass >= 2 && small);
-            if (__all_sync(0xffffffffu, done || !good)) break;
-            static_for<0, NC>([&](auto kk) {
-                constexpr int k = decltype(kk)::value;
-                if (c == k) {
-                    constexpr int i = Packed<DIM>::I(k), j = Packed<DIM>::J(k);
-                    r = fma(-A.a, unscaled_double(y[k], emax), r);
-                    static_for<0, DIM>([&](auto ll) {
-                        constexpr int l = decltype(ll)::value;
-                        constexpr int lj = PackedIndex<DIM>::at(l, j), li = PackedIndex<DIM>::at(l, i);
-                        r = fma(sK[(i * DIM + l) * kT64 + lane], unscaled_double(y[lj], emax), r);
-                        r = fma(sK[(j * DIM + l) * kT64 + lane], unscaled_double(y[li], emax), r);
-                    });
-                }
-            });
-            sR[(1 + ((pass + 1) & 1)) * NC * kT64 + c * kT64 + lane] = r;
-            named_sync<NC * 32>();
-        }
         unsigned fl = 0u;
-        if (!good || !done) {
-            if (!solve_by_elimination<DIM>(sK + lane, sR + lane, A.a, c, &x) && active) fl |= 2u;
-        }
+        if (!refine_solve64<DIM, false>(sK + lane, sKf + lane, sR + lane, A.a, B.a, c, r, &x) && active) fl |= 2u;
         const long long q = (long long)c * A.N + p;
         bool finite = finite64(x);
         if (active) {

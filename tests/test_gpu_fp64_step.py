@@ -83,3 +83,30 @@ def test_systems_beyond_the_refinement(dim, n, kind):
     scale = np.max(np.abs(ref), axis=0)
     assert np.max(np.max(np.abs(got - ref), axis=0)[scale > 0] / scale[scale > 0]) < 1e-11
     assert np.all(got[:, scale == 0] == 0.0)
+
+
+@pytest.mark.parametrize("dim,n", [(2, (40, 3)), (3, (9, 4, 3))])
+@pytest.mark.parametrize("scale", [0.5, 300.0])
+def test_adjoint_of_ordinary_and_indefinite_systems(dim, n, scale):
+    # the transposed point systems through the same refinement and elimination; two steps from a random
+    # stress, every entry of the gradients against the oracle's reverse sweep.  1e-9 of the largest: two reverse steps
+    # through systems of condition up to 1e5.
+    import torch
+    from oracle import orc
+    from paper_2411_17294_gb300 import tfs
+    alpha, dt, m, steps = 0.5, 1e-2, 6, 2
+    mu, w = table(alpha, dt, m)
+    _, kap, sigma0 = fields(dim, n, 3)
+    kap = kap * scale
+    lam = np.random.default_rng(9).normal(size=sigma0.shape)
+    prob = orc.Problem(dim=dim, n=n, alpha=alpha, Wi=0.9, beta=0.5, dt=dt, mu=mu, w=w)
+    ref = orc.gradients(prob, sigma0, kap, None, steps, lam)
+    s = tfs.Solver(dim, n, alpha, 0.9, 0.5, dt, m=m, precision=tfs.TFS_FP64, mu=mu, w=w, transport=False)
+    t = lambda a: torch.as_tensor(a, dtype=torch.float64, device="cuda").contiguous()
+    s.set_state(t(sigma0))
+    kt = t(kap)
+    g = s.backward_run(t(lam), s.run(steps, kt), kt)
+    s.close()
+    for got, want in ((g[0].cpu().numpy(), ref["sigma0"]), (g[1].cpu().numpy(), ref["kappa"]),
+                      (np.array(g[2]), np.array(ref["Wi"])), (np.array(g[3]), np.array(ref["beta"]))):
+        assert np.max(np.abs(got - want)) < 1e-9 * np.max(np.abs(want))

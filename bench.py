@@ -496,7 +496,7 @@ NS_COUPLED = dict(name="coupled Navier-Stokes projection + stress step, 2D perio
 
 def ns_coupled_record(dev, steps: int = 10, warmup: int = 3):
     """The coupled step in the paper's order (Section 4.1): the velocity from the
-    stress at t_n by the projection step (tfs_ns_step: 11 FFTs of 1024^2 and the
+    stress at t_n by the projection step (tfs_ns_step: 5 FFTs of 1024^2 and the
     per-mode Poisson and Helmholtz solves), then the stress step with that
     velocity.  The initial velocity is the spectral field scaled to 0.3 of the
     explicit transport's limit.  Times per step of both parts (CUDA events)."""

@@ -4,8 +4,8 @@
 //
 // Bound.  FP64 runs at about 2 operations per clock and SM on this GPU
 // (0.5 - 0.6 T/s), so the step is bound by the number of FP64 instructions, not
-// by its bytes: 4 per (mode, component) and about 280 (3D) or 70 (2D) per point
-// for the point system.  Hence
+// by its bytes: 4 per (mode, component) here and about 160 (3D) or 66 (2D) per
+// point for the rest (an FP64 elimination alone takes 250 in 3D).  Hence
 //   - Q'_j = x - y/4 instead of Q_j = b1 x + b2 y = -2 Q'_j, with the power of two
 //     in the constants (-2 eta_j, 2 c_j): one FMA for Q', one for the history
 //     sum, two for the push-forward, and bitwise the same values (5 before);

@@ -7,6 +7,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <cmath>
 #include <new>
 #include <vector>
@@ -159,7 +160,12 @@ Cplx stencil_symbol(int stencil, double theta) {
 // The contour samples of W and of the factor G of the stencil symbol, on |zeta| = 1
 // refined geometrically towards phi = 0 (zeta = 1).
 struct Contour {
+    static constexpr size_t kBlock = 16;
     std::vector<Cplx> W, G;
+    struct Range {
+        double wi[2], gr[2], gi[2];   // least and greatest Im W, Re G, Im G of kBlock samples
+    };
+    std::vector<Range> ranges;
 };
 
 Contour stability_contour(const tfs_ctx* h) {
@@ -195,31 +201,25 @@ Contour stability_contour(const tfs_ctx* h) {
         C.W[k] = w;
         C.G[k] = ext;
     }
+    auto widen = [](double r[2], double v, bool first) {
+        r[0] = first || v < r[0] ? v : r[0];
+        r[1] = first || v > r[1] ? v : r[1];
+    };
+    C.ranges.resize((K + Contour::kBlock - 1) / Contour::kBlock);
+    for (size_t k = 0; k < K; ++k) {
+        Contour::Range& r = C.ranges[k / Contour::kBlock];
+        const bool first = k % Contour::kBlock == 0;
+        widen(r.wi, C.W[k].im, first);
+        widen(r.gr, C.G[k].re, first);
+        widen(r.gi, C.G[k].im, first);
+        // a block with such a sample is never passed over (no comparison with a NaN holds)
+        if (!std::isfinite(C.W[k].re + C.W[k].im + C.G[k].re + C.G[k].im)) r.wi[0] = r.wi[1] = NAN;
+    }
     return C;
 }
 
-// Winding number about the origin of the closed polygon f = W + t d G: signed
-// crossings of the negative real axis, each segment turning by less than pi
-// (the sum of the segments' principal angles, without an arctangent each).
-bool winding_zero(const Contour& C, const Cplx& d, double t) {
-    const Cplx ls{t * d.re, t * d.im};
-    const size_t K = C.W.size();
-    int wind = 0;
-    Cplx a = cadd(C.W[K - 1], cmul(ls, C.G[K - 1]));
-    for (size_t k = 0; k < K; ++k) {
-        const Cplx f = cadd(C.W[k], cmul(ls, C.G[k]));
-        const bool up = f.im >= 0.0, was_up = a.im >= 0.0;
-        if (up != was_up) {
-            const double cross = a.re * f.im - f.re * a.im;
-            if (was_up && cross > 0.0) ++wind;
-            if (up && cross < 0.0) --wind;
-        }
-        a = f;
-    }
-    return wind == 0;
-}
-
-// The same number from the sum of the segments' principal angles.
+// Winding number about the origin of the closed polygon f = W + t d G, from the
+// sum of the segments' principal angles.
 bool winding_zero_angles(const Contour& C, const Cplx& d, double t) {
     const Cplx ls{t * d.re, t * d.im};
     const size_t K = C.W.size();
@@ -234,76 +234,65 @@ bool winding_zero_angles(const Contour& C, const Cplx& d, double t) {
     return !(std::fabs(wind) > M_PI);
 }
 
-// An estimate of the smallest t > 0 at which a segment of some polygon passes
-// through the origin: along a segment both W and G are linear, so the
-// condition Im(W conj(d G)) = 0 is a quadratic, and t = -Re(W / (d G)) there.
-double first_crossing(const Contour& C, const std::vector<Cplx>& dirs) {
+// The same number without an arctangent per segment: signed crossings of the negative real
+// axis, each segment turning the way the sign of its quotient says.  Few
+// segments change the sign of the imaginary part: blocks of samples whose ranges
+// leave it one sign are passed over (rounding is monotone, so the sums at the ranges' ends bound
+// the samples' sums).
+bool winding_zero(const Contour& C, const Cplx& d, double t) {
+    const Cplx ls{t * d.re, t * d.im};
     const size_t K = C.W.size();
-    double best = 1e300;
-    for (const Cplx& d : dirs) {
-        Cplx w0 = C.W[K - 1], g0 = cmul(d, C.G[K - 1]);
-        double c0 = w0.im * g0.re - w0.re * g0.im;
-        for (size_t k = 0; k < K; ++k) {
-            const Cplx w1 = C.W[k], g1 = cmul(d, C.G[k]);
-            const double c1 = w1.im * g1.re - w1.re * g1.im;
-            if ((c0 >= 0.0) != (c1 >= 0.0)) {
-                const Cplx dw = csub(w1, w0), dg = csub(g1, g0);
-                double lo = 0.0, hi = 1.0;   // the sign changes once in between
-                for (int it = 0; it < 50; ++it) {
-                    const double x = 0.5 * (lo + hi);
-                    const Cplx w{w0.re + x * dw.re, w0.im + x * dw.im}, g{g0.re + x * dg.re, g0.im + x * dg.im};
-                    if ((w.im * g.re - w.re * g.im >= 0.0) == (c0 >= 0.0)) lo = x;
-                    else hi = x;
-                }
-                const Cplx w{w0.re + lo * dw.re, w0.im + lo * dw.im}, g{g0.re + lo * dg.re, g0.im + lo * dg.im};
-                const double t = -(w.re * g.re + w.im * g.im) / (g.re * g.re + g.im * g.im);
-                if (t > 0.0 && t < best) best = t;
+    auto im = [&](double wi, double gr, double gi) { return wi + (ls.re * gi + ls.im * gr); };
+    auto upper = [&](size_t k) { return im(C.W[k].im, C.G[k].re, C.G[k].im) >= 0.0; };
+    auto at = [&](size_t k) { return cadd(C.W[k], cmul(ls, C.G[k])); };
+    const int pr = ls.im < 0.0, pi = ls.re < 0.0;   // which end of a range is its product's least
+    int wind = 0;
+    bool was_up = upper(K - 1);
+    for (size_t b = 0; b < C.ranges.size(); ++b) {
+        const Contour::Range& r = C.ranges[b];
+        if (was_up ? im(r.wi[0], r.gr[pr], r.gi[pi]) >= 0.0 : im(r.wi[1], r.gr[1 - pr], r.gi[1 - pi]) < 0.0) continue;
+        const size_t end = std::min(K, (b + 1) * Contour::kBlock);
+        for (size_t k = b * Contour::kBlock; k < end; ++k) {
+            const bool up = upper(k);
+            if (up != was_up) {
+                const double turn = cdiv(at(k), at(k == 0 ? K - 1 : k - 1)).im;
+                // exactly through the origin, or not a number: as the angles have it
+                if (!(turn > 0.0 || turn < 0.0)) return winding_zero_angles(C, d, t);
+                if (was_up && turn > 0.0) ++wind;
+                if (up && turn < 0.0) --wind;
             }
-            w0 = w1;
-            g0 = g1;
-            c0 = c1;
+            was_up = up;
         }
     }
-    return best;
+    return wind == 0;
 }
 
 // Largest t such that f = W + t d G keeps winding number 0 about the origin on
-// |zeta| = 1 for every direction d in `dirs`: doubling, then bisection.  The
-// search visits the points that first_crossing() predicts and only its last
-// bracket is tested on the polygons (stable below, unstable above: the test is
-// monotone in t, so these two decide every earlier comparison); if the bracket
-// does not hold, every point is tested.  An explicit-transport run from a new
-// handle pays for this once before its first step: 310 ms with every point
-// tested (about 55 of them, an arctangent per segment), 4 ms this way (the mean
-// over 648 tables, stencils and grids, with the same bounds).  `marginal`: the
-// polygon passes the origin at rounding distance whatever t (purely imaginary
-// symbols with W = delta), where only the full search by angles is repeatable.
-double stability_bound(const Contour& C, const std::vector<Cplx>& dirs, bool marginal) {
-    auto tested = [&](double t) {
+// |zeta| = 1 for every direction d in `dirs`: doubling, then bisection, every point of it tested.
+// (The test is not monotone in t: with the central stencil, whose symbols are imaginary
+// as W nearly is about zeta = 1, and in the paper's variable, where f vanishes at zeta = 1,
+// polygons pass the origin at rounding distance, and single t far below the bound are unstable
+// by a rounding error.)  An explicit-transport run from a new handle pays for the search once
+// before its first step: 2 ms with the upwind stencil, 7 ms with the central one (270 ms with an
+// arctangent per segment; the same bounds over 10000 tables, stencils and forms).
+double stability_bound(const Contour& C, const std::vector<Cplx>& dirs) {
+    auto stable = [&](double t) {
         for (const Cplx& d : dirs)
-            if (!(marginal ? winding_zero_angles(C, d, t) : winding_zero(C, d, t))) return false;
+            if (!winding_zero(C, d, t)) return false;
         return true;
     };
-    auto search = [&](auto&& stable, double& lo, double& hi) {
-        lo = 1e-12;
-        hi = 1e-6;
-        if (!stable(lo)) return false;
-        while (stable(hi) && hi < 1e6) {
-            lo = hi;
-            hi *= 2.0;
-        }
-        for (int it = 0; it < 50 && hi - lo > 1e-7 * hi; ++it) {
-            const double mid = 0.5 * (lo + hi);
-            if (stable(mid)) lo = mid;
-            else hi = mid;
-        }
-        return true;
-    };
-    double lo, hi;
-    if (marginal) return search(tested, lo, hi) ? lo : 0.0;
-    const double edge = first_crossing(C, dirs);
-    if (search([&](double t) { return t < edge; }, lo, hi) && tested(lo) && !tested(hi)) return lo;
-    return search(tested, lo, hi) ? lo : 0.0;
+    double lo = 1e-12, hi = 1e-6;
+    if (!stable(lo)) return 0.0;
+    while (stable(hi) && hi < 1e6) {
+        lo = hi;
+        hi *= 2.0;
+    }
+    for (int it = 0; it < 50 && hi - lo > 1e-7 * hi; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (stable(mid)) lo = mid;
+        else hi = mid;
+    }
+    return lo;
 }
 
 // Courant check.  With lambda_tot = dt sum_a |u_a|/h_a and nu_tot = eps dt sum_a 1/h_a^2
@@ -318,13 +307,10 @@ void ensure_limits(tfs_ctx* h) {
     if (h->lim_valid) return;
     const int nth = 240;
     std::vector<Cplx> S;
-    // half the circle: the symbol at 2 pi - theta is the conjugate, W and G
-    // are conjugate-symmetric, and the conjugate polygon winds alike
-    const bool marginal = h->paper() && h->stencil == TFS_STENCIL_CENTRAL2;
-    for (int t = 1; t <= (marginal ? nth - 1 : nth / 2); ++t) S.push_back(stencil_symbol(h->stencil, 2 * M_PI * t / nth));
+    for (int t = 1; t < nth; ++t) S.push_back(stencil_symbol(h->stencil, 2 * M_PI * t / nth));
     const Contour C = stability_contour(h);
-    h->lam_star = stability_bound(C, S, marginal);
-    h->z_star = stability_bound(C, std::vector<Cplx>{Cplx{1.0, 0.0}}, false);
+    h->lam_star = stability_bound(C, S);
+    h->z_star = stability_bound(C, std::vector<Cplx>{Cplx{1.0, 0.0}});
     h->lim_valid = true;
 }
 

@@ -92,8 +92,12 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 // and x = y0 + y1 + ..., each y the FP32 solution for the residual so far, each thread
 // forming its component's FP64 residual.  With contraction q per pass the error after
 // y2 is |y2| q: q < 2^-18 leaves it below the last bit, and then |y2| is below 2^-36 |x|;
-// otherwise further passes follow.  Points whose refinement does not contract, or whose
-// numbers leave the FP32 range, go to FP64 elimination with partial pivoting.
+// otherwise further passes follow.  FP64 elimination with partial pivoting takes over where
+// the refinement does not contract, where a right-hand side or solution is outside the FP32
+// images' range, where the matrix is (its entries' sum from 2^64 up: what a y below the FP32
+// normal numbers contributes to a residual is then not negligible any more, and from 2^128 the
+// factors are not finite), and for a component whose own residual is so far below the point's
+// others (2^-126) that its image or its y vanishes.
 template <int DIM, bool TRANSPOSED>
 __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sKf, double* sR, double a, float af,
                                                int c, double r, double* out) {
@@ -114,10 +118,21 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             F.a[ro][k] = v;
         });
     });
+    float entries = 0.0f;
+    static_for<0, NC>([&](auto rr) {
+        constexpr int ro = decltype(rr)::value;
+        float off = 0.0f;   // as row_dominant() forms it
+        static_for<0, NC>([&](auto kk) {
+            constexpr int k = decltype(kk)::value;
+            if (k != ro) off += fabsf(F.a[ro][k]);
+        });
+        entries += off + fabsf(F.a[ro][ro]);
+    });
     bool good = row_dominant<NC>(F) ? lu32_factor_nopivot<NC>(F, 1e-30f) : lu32_factor<NC>(F, 1e-30f);
+    good = good && entries < 18446744073709551616.0f;   // false for a NaN
     int e0 = 0;
     constexpr int kMaxPass = 8;
-    bool done = false;
+    bool done = false, lost = false;
     double x = 0.0;
     for (int pass = 0; pass < kMaxPass; ++pass) {
         const double* rb = pass == 0 ? sR : sR + (1 + (pass & 1)) * NC * kT64;
@@ -137,6 +152,11 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             y[k] = scaled_float(rv[k], emax);
         }
         if (pass == 0) good = good && emax < 0x7ff && (emax > 200 || zero);
+        float own = 0.0f;
+        static_for<0, NC>([&](auto kk) {
+            constexpr int k = decltype(kk)::value;
+            if (c == k) own = y[k];
+        });
         lu32_solve<NC>(F, y);
         unsigned ymax = 0u;
 #pragma unroll
@@ -146,11 +166,14 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             good = good && ymax < 0x7f800000u && ey - 127 < 0x7ff;
             e0 = ey;
         }
-        const bool small = ymax == 0u || ey <= e0 - 36;
+        const bool small = ymax != 0u && ey <= e0 - 36;
         static_for<0, NC>([&](auto kk) {
             constexpr int k = decltype(kk)::value;
             // a point's passes are its own, whatever the other points of its tile still need
-            if (c == k && !done) x += unscaled_double(y[k], emax);
+            if (c == k && !done) {
+                x += unscaled_double(y[k], emax);
+                lost = lost || (!zero64(r) && (own == 0.0f || (__float_as_uint(y[k]) & 0x7fffffffu) < 0x00800000u));
+            }
         });
         done = done || zero || (pass >= 2 && small);
         // the same data in every warp of the tile: they leave together
@@ -180,7 +203,7 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
         named_sync<NC * 32>();
     }
     bool ok = true;
-    if (!good || !done) ok = solve_by_elimination<DIM>(sK, sR, a, c, TRANSPOSED, &x);
+    if (!good || !done || lost) ok = solve_by_elimination<DIM>(sK, sR, a, c, TRANSPOSED, &x);
     *out = x;
     return ok;
 }

@@ -63,8 +63,7 @@ __host__ __device__ constexpr size_t smem64_bytes(int m, int groups) {
 
 // Products of the step's scalars, formed once on the host.
 struct Step64 {
-    double scale;      // dt (the paper's variable: dt xi): what kappa* is scaled by
-    double src;        // dt G g / scale
+    double src;        // G g (kappa* comes with dt)
     double g6[3];      // dt / (6 h_a)
     double lap[3];     // eps dt / h_a^2
     float inv_h[3];
@@ -172,9 +171,10 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
     double* sQ = sm64;                          // Q'_j [m][NC][32]
     double* sH = sQ + (size_t)m * NC * kT64;    // partial history sums [G][NC][32]
     double* sR = sH + G * NC * kT64;            // right-hand side, then two buffers of residuals [3][NC][32]
-    double* sK = sR + 3 * NC * kT64;            // dt kappa* (the paper's variable: dt xi kappa*) [DD][32]
+    double* sK = sR + 3 * NC * kT64;            // dt kappa* [DD][32]
     double* sC = sK + DD * kT64;                // stencil coefficients
-    float* sKf = reinterpret_cast<float*>(sC + Shape64<DIM>::kCoef * kT64);   // sK in FP32
+    // dt kappa* in FP32 (the paper's variable: dt xi kappa*, the operator's)
+    float* sKf = reinterpret_cast<float*>(sC + Shape64<DIM>::kCoef * kT64);
     const long long t0 = (long long)blockIdx.x * kT64;
     const long long p = t0 + lane;
     const bool active = p < A.N;
@@ -184,9 +184,9 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
     // ---- velocity gradient entries and stencil coefficients, spread over the warps
     for (int k = w; k < DD; k += NC * G) {
         const long long q = (long long)k * A.N + pc;
-        const double v = B.scale * fma(2.0, A.kap_n[q], -A.kap_nm1[q]);
+        const double v = A.dt * fma(2.0, A.kap_n[q], -A.kap_nm1[q]);
         sK[k * kT64 + lane] = v;
-        sKf[k * kT64 + lane] = (float)v;
+        sKf[k * kT64 + lane] = (float)(PAPER ? A.xi * v : v);
     }
     if (TR == kInStep && w == NC * G - 1) {
         double u[DIM];
@@ -269,8 +269,7 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
             for (int l = 0; l < DIM; ++l)
                 lh = fma(sK[(ci * DIM + l) * kT64 + lane], hat(l, cj),
                          fma(hat(ci, l), sK[(cj * DIM + l) * kT64 + lane], lh));
-            // (sK carries dt xi; A.eta holds 1/xi in this variable)
-            r = fma(2.0, A.sig_n[q], -0.5 * A.sig_nm1[q]) - A.dt * A.inv_wi * H + fma(B.src, ks, A.eta * lh);
+            r = fma(2.0, A.sig_n[q], -0.5 * A.sig_nm1[q]) - A.dt * A.inv_wi * H + fma(B.src, ks, lh);
             if (TR == kFromPrepass) r -= A.trans[q];
         } else {
             s0 = has_s0 ? A.sigma0[q] : 0.0;
@@ -282,7 +281,9 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
     __syncthreads();
     if (grp == 0) {
         unsigned fl = 0u;
-        if (!refine_solve64<DIM, false>(sK + lane, sKf + lane, sR + lane, A.a, B.a, c, r, &x) && active) fl |= 2u;
+        if (!refine_solve64<DIM, false, PAPER>(sK + lane, sKf + lane, sR + lane, A.a, B.a, c, r, &x, PAPER ? A.xi : 1.0) &&
+            active)
+            fl |= 2u;
         const long long q = (long long)c * A.N + p;
         bool finite = finite64(x);
         if (active) {
@@ -336,8 +337,7 @@ cudaError_t launch64(const FwdArgs<double>& a, const LaunchCfg& cfg, long long t
     if (e != cudaSuccess) return e;
     const size_t dyn = smem64_bytes<DIM>(cfg.classic ? 0 : a.m, G);
     Step64 b;
-    b.scale = PAPER ? a.dt * a.xi : a.dt;
-    b.src = PAPER ? a.G * a.g / a.xi : a.G * a.g;
+    b.src = a.G * a.g;
     for (int i = 0; i < 3; ++i) {
         b.g6[i] = a.dt * a.inv_h[i] / 6.0;
         b.lap[i] = a.eps * a.dt * a.inv_h[i] * a.inv_h[i];
@@ -387,7 +387,6 @@ cudaError_t launch_forward_f64(const FwdArgs<double>& args, const LaunchCfg& cfg
         if (e != cudaSuccess) return e;
     }
     FwdArgs<double> a = args;
-    if (cfg.paper) a.eta = 1.0 / a.xi;
     for (int j = 0; j < a.m; ++j) {   // Q = -2 Q'
         a.mc.c[j] *= 2.0;
         a.mc.eta[j] *= -2.0;

@@ -51,11 +51,11 @@ struct PackedIndex {
     }
 };
 
-// The point system by FP64 Gaussian elimination (K scaled as in the kernel):
-// component c of M^-1 R.  Returns false when a pivot vanishes.
+// The point system M = a I - scale L(K) by FP64 Gaussian elimination: component c of
+// M^-1 R.  Returns false when a pivot vanishes.
 template <int DIM>
-__device__ __noinline__ bool solve_by_elimination(const double* sK, const double* sR, double a, int c, bool transposed,
-                                                   double* out) {
+__device__ __noinline__ bool solve_by_elimination(const double* sK, const double* sR, double a, double scale, int c,
+                                                   bool transposed, double* out) {
     constexpr int NC = Packed<DIM>::NC;
     double K[3][3], x[NC], M[NC][NC];
 #pragma unroll
@@ -64,7 +64,7 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
         for (int j = 0; j < DIM; ++j) K[i][j] = sK[(i * DIM + j) * kT64];
 #pragma unroll
     for (int r = 0; r < NC; ++r) x[r] = sR[r * kT64];
-    assemble_M<DIM>(K, a, 1.0, M);
+    assemble_M<DIM>(K, a, scale, M);
     if (transposed) {
 #pragma unroll
         for (int i = 0; i < NC; ++i)
@@ -83,9 +83,9 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
     return ok;
 }
 
-// Component c of M^-1 R (TRANSPOSED: M^-T R), M = a I - L(K), for this lane's point; every
-// lane of the NC warps of the tile calls it.  sK, sKf: K scaled by the operator's dt, in
-// FP64 and FP32 [d*d][32]; sR: R [NC][32] followed by two buffers of that size for the residuals (all at this
+// Component c of M^-1 R (TRANSPOSED: M^-T R), M = a I - scale L(K), for this lane's point; every
+// lane of the NC warps of the tile calls it.  sK: K in FP64 [d*d][32]; sKf: scale K in FP32
+// (SCALED false: scale is 1); sR: R [NC][32] followed by two buffers of that size for the residuals (all at this
 // lane); r: this thread's entry of R.  Returns false when a pivot vanishes.
 //
 // The warps factor the tile's 32 matrices in FP32, each for itself (the FP32 pipe is idle),
@@ -98,9 +98,10 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 // normal numbers contributes to a residual is then not negligible any more, and from 2^128 the
 // factors are not finite), and for a component whose own residual is so far below the point's
 // others (2^-126) that its image or its y vanishes.
-template <int DIM, bool TRANSPOSED>
+template <int DIM, bool TRANSPOSED, bool SCALED = false>
 __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sKf, double* sR, double a, float af,
-                                               int c, double r, double* out) {
+                                               int c, double r, double* out, double scale = 1.0) {
+    static_assert(!(TRANSPOSED && SCALED), "the transposed systems take K scaled");
     constexpr int NC = Packed<DIM>::NC;
     LU32<NC> F;
     static_for<0, NC>([&](auto rr) {
@@ -183,27 +184,29 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             if (c == k) {
                 constexpr int i = Packed<DIM>::I(k), j = Packed<DIM>::J(k);
                 r = fma(-a, unscaled_double(y[k], emax), r);
+                double q = SCALED ? 0.0 : r;
                 static_for<0, DIM>([&](auto ll) {
                     constexpr int l = decltype(ll)::value;
                     constexpr int lj = PackedIndex<DIM>::at(l, j), li = PackedIndex<DIM>::at(l, i);
                     if constexpr (!TRANSPOSED) {
-                        r = fma(sK[(i * DIM + l) * kT64], unscaled_double(y[lj], emax), r);
-                        r = fma(sK[(j * DIM + l) * kT64], unscaled_double(y[li], emax), r);
+                        q = fma(sK[(i * DIM + l) * kT64], unscaled_double(y[lj], emax), q);
+                        q = fma(sK[(j * DIM + l) * kT64], unscaled_double(y[li], emax), q);
                     } else {
                         // (L^T y)_ij = sum_l K_li Y_lj + K_lj Y_li (once for i = j), Y symmetric
                         // with the diagonal doubled
-                        r = fma(sK[(l * DIM + i) * kT64], unscaled_double(l == j ? 2.0f * y[lj] : y[lj], emax), r);
+                        q = fma(sK[(l * DIM + i) * kT64], unscaled_double(l == j ? 2.0f * y[lj] : y[lj], emax), q);
                         if constexpr (i != j)
-                            r = fma(sK[(l * DIM + j) * kT64], unscaled_double(l == i ? 2.0f * y[li] : y[li], emax), r);
+                            q = fma(sK[(l * DIM + j) * kT64], unscaled_double(l == i ? 2.0f * y[li] : y[li], emax), q);
                     }
                 });
+                r = SCALED ? fma(scale, q, r) : q;
             }
         });
         sR[(1 + ((pass + 1) & 1)) * NC * kT64 + c * kT64] = r;
         named_sync<NC * 32>();
     }
     bool ok = true;
-    if (!good || !done || lost) ok = solve_by_elimination<DIM>(sK, sR, a, c, TRANSPOSED, &x);
+    if (!good || !done || lost) ok = solve_by_elimination<DIM>(sK, sR, a, scale, c, TRANSPOSED, &x);
     *out = x;
     return ok;
 }

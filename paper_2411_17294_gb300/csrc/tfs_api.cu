@@ -160,7 +160,7 @@ Cplx stencil_symbol(int stencil, double theta) {
 // The contour samples of W and of the factor G of the stencil symbol, on |zeta| = 1
 // refined geometrically towards phi = 0 (zeta = 1).
 struct Contour {
-    static constexpr size_t kBlock = 16;
+    static constexpr size_t kBlock = 32;
     std::vector<Cplx> W, G;
     struct Range {
         double wi[2], gr[2], gi[2];   // least and greatest Im W, Re G, Im G of kBlock samples
@@ -273,12 +273,18 @@ bool winding_zero(const Contour& C, const Cplx& d, double t) {
 // as W nearly is about zeta = 1, and in the paper's variable, where f vanishes at zeta = 1,
 // polygons pass the origin at rounding distance, and single t far below the bound are unstable
 // by a rounding error.)  An explicit-transport run from a new handle pays for the search once
-// before its first step: 2 ms with the upwind stencil, 7 ms with the central one (270 ms with an
-// arctangent per segment; the same bounds over 10000 tables, stencils and forms).
+// before its first step: 2 ms with the upwind stencil, 5 ms with the central one (270 ms with an
+// arctangent per segment; the same bounds over 10400 tables in both forms and stencils).
 double stability_bound(const Contour& C, const std::vector<Cplx>& dirs) {
+    size_t first = 0;   // the direction that failed last: most likely the next to
     auto stable = [&](double t) {
-        for (const Cplx& d : dirs)
-            if (!winding_zero(C, d, t)) return false;
+        for (size_t i = 0; i < dirs.size(); ++i) {
+            const size_t k = (first + i) % dirs.size();
+            if (!winding_zero(C, dirs[k], t)) {
+                first = k;
+                return false;
+            }
+        }
         return true;
     };
     double lo = 1e-12, hi = 1e-6;

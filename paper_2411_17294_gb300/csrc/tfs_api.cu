@@ -894,7 +894,7 @@ cudaError_t back_resident(const tfs_ctx* h, int start, int end, const void* grad
     a.N = h->N;
     a.m = h->m;
     a.mc = h->mcf;
-    a.eta = split_f2(h->eta);
+    a.eta = h->eta;
     a.a = (float)(h->eta + h->dt / h->Wi);
     a.dt = (float)h->dt;
     const double G = (1.0 - h->beta) / (h->Wi * h->Re);
@@ -910,7 +910,7 @@ cudaError_t back_resident(const tfs_ctx* h, int start, int end, const void* grad
         for (int k = 0; k < a.steps; ++k) {
             const double g = g_alpha(h, top - 1 - k);
             a.src[k] = (float)(h->dt * G * g);
-            a.dtg[k] = split_f2(h->dt * g);
+            a.dtg[k] = h->dt * g;
         }
         e = launch_resident_back(a, h->dim, s);
         top = first;

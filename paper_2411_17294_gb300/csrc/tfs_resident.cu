@@ -6,8 +6,11 @@
 // modes to memory between steps: thread (point, component) keeps both levels of
 // its m modes in registers (64 at m = 32) and takes step after step with the
 // arithmetic of the single step (tfs_forward.cu) and of its adjoint
-// (tfs_adjoint.cu), operation for operation, so that every stress and every
-// adjoint value is bitwise the one that stepping gives.  Per step a tile of 32
+// (tfs_adjoint.cu), operation for operation, so that every stress, adjoint mode and
+// adjoint of a right-hand side is bitwise the one that stepping gives.  The gradients are
+// their sums over the steps, which stepping adds up in FP64 and a run in three floats
+// (no less accurate; the FP64 additions took 4.8 us per reverse step at 2D 512^2, these
+// 1 us more than two floats).  Per step a tile of 32
 // points exchanges only its right-hand sides and solutions through shared
 // memory; the point matrix is factored once.
 //
@@ -17,8 +20,8 @@
 // tile, which rotates with the tile so that the solves spread over the SM's
 // schedulers.  Nothing but one stress row per step and, per launch, the mode levels moves:
 // a single step is bound by 3 words per (mode, component) from HBM.  Measured at 2D
-// 512^2, m = 32, 100 steps: 15.7 us per step against 49 for tfs_step, 13.1 us per
-// reverse step against 77; a training pass (forward and gradients) 19.2 -> 3.4 ms, of which
+// 512^2, m = 32, 100 steps: 15.7 us per step against 49 for tfs_step, 14.1 us per
+// reverse step against 77; a training pass (forward and gradients) 19.2 -> 3.5 ms, of which
 // 4.9 ms are the segments' recomputation that stored stresses make unnecessary.
 // Tried and not kept: one mode sweep per block of eight steps with the steps' own drives convolved
 // by scalar weights (4.5 ms; smaller rounding errors, but not the values that stepping gives).
@@ -181,18 +184,29 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_run_kernel(const
     }
 }
 
-// a + v and a + w v (w = hi + lo), compensated
-__device__ __forceinline__ void acc_add(f2& a, float v) {
-    const f2 t = two_sum_f2(a.hi, v);
-    a.hi = t.hi;
-    a.lo = __fadd_rn(a.lo, t.lo);
-}
-__device__ __forceinline__ void acc_dot(f2& a, F2c w, float v) {
-    const f2 pr = two_prod(w.hi, v);
-    const f2 t = two_sum_f2(a.hi, pr.hi);
-    a.hi = t.hi;
-    a.lo = __fadd_rn(a.lo, __fadd_rn(t.lo, __fmaf_rn(w.lo, v, pr.lo)));
-}
+// A sum of floats to at least the accuracy of FP64 additions, off the FP64 pipe
+// (1/64 of the FP32 rate): the errors of the first float's additions, exact by TwoSum, are
+// summed in a second, and those of the second's in a third (72 bits; sums do not underflow).
+struct f3 {
+    float a, b, c;
+    __device__ __forceinline__ void add(float v) {
+        const f2 t = two_sum_f2(a, v);
+        a = t.hi;
+        add_small(t.lo);
+    }
+    // of the order of a rounding error of the sum
+    __device__ __forceinline__ void add_small(float v) {
+        const f2 t = two_sum_f2(b, v);
+        b = t.hi;
+        c = __fadd_rn(c, t.lo);
+    }
+    // the sum as hi + lo, lo below an ulp of hi or nearly so
+    __device__ __forceinline__ void value(double& hi, double& lo) const {
+        hi = (double)a + (double)b;
+        lo = ((double)a - hi) + (double)b + (double)c;   // |a| >= |b|
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
 
 template <int DIM, int MM>
 __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(const ResidentBack A) {
@@ -241,9 +255,10 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
         if (!lu32_factor<NC>(F, 1e-30f)) fl |= 2u;
         sF.put(F, lane);
     }
-    f2 gs{0.0f, 0.0f}, gk[kPer], sig_sum{0.0f, 0.0f}, sym_sum{0.0f, 0.0f};
+    f3 l_sum{0.0f, 0.0f, 0.0f}, s_sum{0.0f, 0.0f, 0.0f}, gk[kPer];   // of lamR, S, dJ/dkappa
+    double sig_sum = 0.0, sym_sum = 0.0;
 #pragma unroll
-    for (int e = 0; e < kPer; ++e) gk[e] = f2{0.0f, 0.0f};
+    for (int e = 0; e < kPer; ++e) gk[e] = f3{0.0f, 0.0f, 0.0f};
 #pragma unroll 1
     for (int k = 0; k < A.steps; ++k) {
         const int n = A.steps - 1 - k;
@@ -280,8 +295,8 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
                 sig_dot = __fmaf_rn(lam[r], sSig[k & 1][r][lane], sig_dot);
                 sL[r][lane] = lam[r];
             }
-            acc_add(sig_sum, sig_dot);
-            acc_dot(sym_sum, A.dtg[k], sym_dot);
+            sig_sum += (double)sig_dot;
+            sym_sum = fma(A.dtg[k], (double)sym_dot, sym_sum);
         }
         __syncthreads();
         const float l = sL[c][lane];
@@ -289,10 +304,10 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
             constexpr int j = decltype(jj)::value;
             x[j] = __fmaf_rn(-A.mc.eta_hi[j], l, x[j]);
         });
-        acc_dot(gs, A.eta, l);
+        l_sum.add(l);
         if (!last) {
-            acc_add(gs, -ss);
-            gs.lo = __fadd_rn(gs.lo, comp);
+            s_sum.add(ss);
+            s_sum.add_small(-comp);
         }
         // dJ/dkappa_ab += dt sum_s Lam_as sigma_bs + dt G g Lam_ab, Lam symmetric with doubled diagonal
 #pragma unroll
@@ -308,7 +323,7 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
                     g = __fmaf_rn(a == s ? 2.0f * la : la, sSig[k & 1][at(b, s)][lane], g);
                 }
                 const float lab = sL[at(a, b)][lane];
-                acc_add(gk[e], __fmaf_rn(A.dt, g, A.src[k] * (a == b ? 2.0f * lab : lab)));
+                gk[e].add(__fmaf_rn(A.dt, g, A.src[k] * (a == b ? 2.0f * lab : lab)));
             }
         }
     }
@@ -319,14 +334,17 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
             __stcs(A.ell_prev + base + j * row, x[j]);
             __stcs(A.ell_prev2 + base + j * row, y[j]);
         });
-        A.g_sigma0[(long long)c * N + p] += (double)gs.hi + (double)gs.lo;
+        // sum of eta lamR - S over the steps
+        double lh, ll, sh, sl;
+        l_sum.value(lh, ll);
+        s_sum.value(sh, sl);
+        A.g_sigma0[(long long)c * N + p] += fma(A.eta, lh, -sh) + fma(A.eta, ll, -sl);
 #pragma unroll
         for (int e = 0; e < kPer; ++e)
-            if (c + e * NC < DD) A.g_kap[(long long)(c + e * NC) * N + p] += (double)gk[e].hi + (double)gk[e].lo;
+            if (c + e * NC < DD) A.g_kap[(long long)(c + e * NC) * N + p] += gk[e].value();
     }
     if (c == ws) {
-        const double sd = active ? (double)sig_sum.hi + (double)sig_sum.lo : 0.0;
-        const double sy = active ? (double)sym_sum.hi + (double)sym_sum.lo : 0.0;
+        const double sd = active ? sig_sum : 0.0, sy = active ? sym_sum : 0.0;
         double wi = A.dt_wi2 * sd - A.g_wi * sy, be = -A.inv_wire * sy;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {

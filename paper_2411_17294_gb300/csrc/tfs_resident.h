@@ -38,11 +38,10 @@ struct ResidentBack {
     long long N;
     int m, steps;
     ModeConstsF mc;
-    F2c eta;
     float a, dt;
-    double dt_wi2, g_wi, inv_wire;   // dt/Wi^2, G/Wi, 1/(Wi Re)
+    double eta, dt_wi2, g_wi, inv_wire;   // eta, dt/Wi^2, G/Wi, 1/(Wi Re)
     float src[kRunSteps];            // dt G g_alpha
-    F2c dtg[kRunSteps];              // dt g_alpha
+    double dtg[kRunSteps];           // dt g_alpha
 };
 cudaError_t launch_resident_back(const ResidentBack& a, int dim, cudaStream_t s);
 

@@ -22,6 +22,7 @@
 // The forward modes themselves are never needed: only sigma^{n+1} and kappa.
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "tfs_device.cuh"
@@ -405,9 +406,13 @@ adj_kernel(const AdjArgs<T> A, const int classic, const long long num_tiles, con
 // passes 2 lamE to the adjoint of sigma^n and -lamE to that of sigma^{n-1}.
 // The point p = q - k e_a reads q with its tap k, whose weight is
 // dt u_a(p) / (6 h_a) times a small integer, with the Laplacian's.
+struct F3c {
+    float a, b, c;
+};
 struct GatherScales {
-    double g6[3], lap[3];   // dt / (6 h_a), eps dt / h_a^2
-    F2c g6f[3], lapf[3];    // the same as hi + lo
+    double g6[3], lap[3];           // dt / (6 h_a), eps dt / h_a^2
+    F3c tap[3][4], lapf[3][2];      // g6 times 1, 2, 3, 6 and lap times 1, -2, times 1/unscale
+    double unscale;                 // a power of two
 };
 
 // six times the weight of tap k, 0 where the stencil does not read it
@@ -427,66 +432,117 @@ __device__ __forceinline__ long long neighbour(int v, int off, int n, long long 
     return (long long)(w - v) * stride;
 }
 
-// FP64 storage: all in FP64, two operations per tap shared by the components and
-// one FMA per component.  FP32 storage (lamR holds float values): the sums in
-// double-float on the FP32 pipe (products exact by FMA, TwoSum; 2^-47 of the sum), since the FP64
-// pipe has 1/64 of its rate, added to the FP64 fields at the end.  Thread =
-// point; the x rows of neighbouring threads come from L1.  3D 64^3, FP32 storage: 151 -> 39 us (all in
-// FP64 with its weights formed per tap before); a training pass of 40 steps 19.5 -> 14.6 ms.
-template <typename TU, int DIM>
-__global__ void __launch_bounds__(128) adj_transport_kernel(const AdjArgs<double> A, const GatherScales Q,
-                                                            const TU* __restrict__ lamR, const TU* __restrict__ u,
-                                                            const int stencil) {
-    constexpr int NC = Packed<DIM>::NC;
-    constexpr bool F32 = sizeof(TU) == 4;
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= A.N) return;
+__device__ __forceinline__ bool is_zero(float v) { return v == 0.0f; }
+__device__ __forceinline__ bool is_zero(double v) { return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0; }
+
+// Calls tap(offset of p, axis, k, u_a(p), six times the tap's weight, whether the Laplacian reads it) for every
+// point p whose stencil reads q.
+template <int DIM, typename TU, typename F>
+__device__ __forceinline__ void for_taps(const AdjArgs<double>& A, const TU* __restrict__ u, int stencil, long long q,
+                                         F&& tap) {
     const unsigned qu = (unsigned)q, r1 = qu / (unsigned)A.n0;
     const int co[3] = {(int)(qu % (unsigned)A.n0), (int)(DIM == 3 ? r1 % (unsigned)A.n1 : r1),
                        (int)(DIM == 3 ? r1 / (unsigned)A.n1 : 0)};
     const int nn[3] = {A.n0, A.n1, A.n2};
     const long long st[3] = {1, A.n0, (long long)A.n0 * A.n1};
     const bool diffusion = A.eps != 0.0;
-    double lamE[NC];
-    f2 lamF[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        lamE[c] = 0.0;
-        lamF[c] = f2{0.0f, 0.0f};
-    }
-#pragma unroll
-    for (int ax = 0; ax < DIM; ++ax) {
-#pragma unroll
-        for (int k = -2; k <= 2; ++k) {
-            const long long pnb = q + neighbour(co[ax], -k, nn[ax], st[ax]);
-            const TU ua = __ldg(u + (long long)ax * A.N + pnb);
+    static_for<0, DIM>([&](auto aa) {
+        constexpr int ax = decltype(aa)::value;
+        static_for<0, 5>([&](auto kk) {
+            constexpr int k = decltype(kk)::value - 2;
+            const long long p = q + neighbour(co[ax], -k, nn[ax], st[ax]);
+            const TU ua = __ldg(u + (long long)ax * A.N + p);
             const float w6 = tap_weight(stencil, ua >= (TU)0, k);
-            const float wl = diffusion ? (k == 0 ? 2.0f : (k == 1 || k == -1 ? -1.0f : 0.0f)) : 0.0f;
-            if constexpr (F32) {
-                if ((w6 == 0.0f || ua == 0.0f) && wl == 0.0f) continue;
-                f2 w = f2_mul_f(f2_mul_f(f2{Q.g6f[ax].hi, Q.g6f[ax].lo}, ua), -w6);
-                if (wl != 0.0f) w = f2_add(w, f2{-wl * Q.lapf[ax].hi, -wl * Q.lapf[ax].lo});
+            const bool lap = diffusion && k >= -1 && k <= 1;
+            if ((w6 != 0.0f && !is_zero(ua)) || lap) tap(p, aa, std::integral_constant<int, k>{}, ua, w6, lap);
+        });
+    });
+}
+
+// lamE(q) in FP64: two operations per tap shared by the components and one FMA per component.
+template <int DIM, typename TU>
+__device__ __forceinline__ void gather(const AdjArgs<double>& A, const GatherScales& Q, const TU* __restrict__ lamR,
+                                       const TU* __restrict__ u, int stencil, long long q, double* lamE) {
+    constexpr int NC = Packed<DIM>::NC;
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const float v = __ldg(lamR + (long long)c * A.N + pnb);
-                    const f2 p = two_prod(w.hi, v);
-                    const f2 t = two_sum_f2(lamF[c].hi, p.hi);
-                    lamF[c].hi = t.hi;
-                    lamF[c].lo = __fadd_rn(lamF[c].lo, __fadd_rn(t.lo, __fmaf_rn(w.lo, v, p.lo)));
-                }
-            } else {
-                if (w6 == 0.0f && wl == 0.0f) continue;
-                double w = Q.g6[ax] * ua * (double)-w6;
-                if (wl != 0.0f) w = fma((double)-wl, Q.lap[ax], w);
+    for (int c = 0; c < NC; ++c) lamE[c] = 0.0;
+    for_taps<DIM>(A, u, stencil, q, [&](long long p, auto aa, auto kk, TU ua, float w6, bool lap) {
+        constexpr int ax = decltype(aa)::value, k = decltype(kk)::value;
+        double w = Q.g6[ax] * (double)ua * (double)-w6;
+        if (lap) w = fma(k == 0 ? -2.0 : 1.0, Q.lap[ax], w);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) lamE[c] = fma(w, __ldg(lamR + (long long)c * A.N + pnb), lamE[c]);
+        for (int c = 0; c < NC; ++c) lamE[c] = fma(w, (double)__ldg(lamR + (long long)c * A.N + p), lamE[c]);
+    });
+}
+
+template <int DIM>
+__device__ __noinline__ void gather_out_of_range(const AdjArgs<double>& A, const GatherScales& Q, const float* lamR,
+                                                 const float* u, int stencil, long long q, double* lamE) {
+    gather<DIM, float>(A, Q, lamR, u, stencil, q, lamE);
+}
+
+// FP64 storage: all in FP64.  FP32 storage (lamR and u hold floats): the FP64 pipe's rate, 1/64 of the FP32
+// pipe's, would bound it (104 operations and as many conversions per 3D point), so weights and sums are
+// three floats each, to more than the accuracy of the FP64 form (largest error of a sum, relative to the sum
+// of its products' magnitudes, 1.1e-16 against 4.3e-16; two floats 2.7e-14).  The weights carry a power of two that
+// keeps the products' rounding errors representable for every normal lamR; sums beyond
+// the float range are formed again in FP64.  Thread = point; the x rows of
+// neighbouring threads come from L1.  3D 64^3, FP32 storage: 61 us, against 92 in FP64 with conversions by integer
+// operations, 140 with the FP64 pipe's, and 33 for sums of two floats.
+template <typename TU, int DIM>
+__global__ void __launch_bounds__(128) adj_transport_kernel(const AdjArgs<double> A, const GatherScales Q,
+                                                            const TU* __restrict__ lamR, const TU* __restrict__ u,
+                                                            const int stencil) {
+    constexpr int NC = Packed<DIM>::NC;
+    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= A.N) return;
+    double lamE[NC];
+    if constexpr (sizeof(TU) == 8) {
+        gather<DIM, TU>(A, Q, lamR, u, stencil, q, lamE);
+    } else {
+        f3 s[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c] = f3{0.0f, 0.0f, 0.0f};
+        for_taps<DIM>(A, u, stencil, q, [&](long long p, auto aa, auto kk, float ua, float w6, bool lap) {
+            constexpr int ax = decltype(aa)::value, k = decltype(kk)::value;
+            // -w6 g6 u [+ lap] as three floats
+            const float m = fabsf(w6), us = m == 0.0f ? 0.0f : (w6 > 0.0f ? -ua : ua);
+            const F3c g = m == 1.0f ? Q.tap[ax][0] : (m == 2.0f ? Q.tap[ax][1] : (m == 3.0f ? Q.tap[ax][2] : Q.tap[ax][3]));
+            const f2 p0 = two_prod(g.a, us), p1 = two_prod(g.b, us);
+            const f2 t = two_sum_f2(p0.lo, p1.hi), h = fast_two_sum(p0.hi, t.hi);
+            f3 w{h.hi, h.lo, __fadd_rn(t.lo, __fmaf_rn(g.c, us, p1.lo))};
+            if (lap) {
+                const F3c l = Q.lapf[ax][k == 0 ? 1 : 0];
+                w.add(l.a);
+                w.add_small(l.b);
+                w.c = __fadd_rn(w.c, l.c);
             }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const float v = __ldg(lamR + (long long)c * A.N + p);
+                const f2 a0 = two_prod(w.a, v), a1 = two_prod(w.b, v);
+                s[c].add(a0.hi);
+                s[c].add_small(a0.lo);
+                s[c].add_small(a1.hi);
+                s[c].c = __fadd_rn(s[c].c, __fmaf_rn(w.c, v, a1.lo));
+            }
+        });
+        bool finite = true;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            finite = finite && isfinite(s[c].a + s[c].b + s[c].c);
+            lamE[c] = s[c].value() * Q.unscale;
+        }
+        if (!finite) {
+            double out[NC];
+            gather_out_of_range<DIM>(A, Q, lamR, u, stencil, q, out);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) lamE[c] = out[c];
         }
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         const long long i = (long long)c * A.N + q;
-        if constexpr (F32) lamE[c] = (double)lamF[c].hi + (double)lamF[c].lo;
         A.s1_out[i] = fma(2.0, lamE[c], A.s1_out[i]);
         A.s0_out[i] -= lamE[c];
     }
@@ -543,21 +599,30 @@ cudaError_t launch_adjoint_f32(const AdjArgs<float>& a, const LaunchCfg& cfg, cu
     return cfg.dim == 2 ? launch_adj<float, 2>(a, cfg, s) : launch_adj<float, 3>(a, cfg, s);
 }
 
+// v as three floats
+static F3c split_f3(double v) {
+    const float a = (float)v, b = (float)(v - (double)a);
+    return F3c{a, b, (float)(v - (double)a - (double)b)};
+}
+
 cudaError_t launch_adjoint_transport(const AdjArgs<double>& a, const void* lamR, const void* u, bool is_double,
                                      const LaunchCfg& cfg, cudaStream_t s) {
     const int threads = 128;
     const unsigned blocks = (unsigned)((a.N + threads - 1) / threads);
     GatherScales q;
-    auto split = [](double v) {
-        const float hi = (float)v;
-        return F2c{hi, (float)(v - (double)hi)};
-    };
+    double top = 0.0;
     for (int i = 0; i < 3; ++i) {
         q.g6[i] = a.dt * a.inv_h[i] / 6.0;
         q.lap[i] = a.eps * a.dt * a.inv_h[i] * a.inv_h[i];
-        q.g6f[i] = split(q.g6[i]);
-        q.lapf[i] = split(q.lap[i]);
+        if (i < cfg.dim) top = std::fmax(top, std::fmax(q.g6[i], q.lap[i]));
     }
+    const int up = top > 0.0 && std::isfinite(top) ? 30 - std::ilogb(top) : 0;   // weights of unit velocity near 2^30
+    const double factor[4] = {1.0, 2.0, 3.0, 6.0};
+    for (int i = 0; i < 3; ++i) {
+        for (int j = 0; j < 4; ++j) q.tap[i][j] = split_f3(std::ldexp(factor[j] * q.g6[i], up));
+        for (int j = 0; j < 2; ++j) q.lapf[i][j] = split_f3(std::ldexp((j ? -2.0 : 1.0) * q.lap[i], up));
+    }
+    q.unscale = std::ldexp(1.0, -up);
     if (cfg.dim == 2) {
         if (is_double)
             adj_transport_kernel<double, 2><<<blocks, threads, 0, s>>>(a, q, (const double*)lamR, (const double*)u, cfg.stencil);

@@ -353,6 +353,30 @@ __device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
     return fast_two_sum(p.hi, p.lo);
 }
 
+// A sum of floats to at least the accuracy of FP64 additions, off the FP64 pipe
+// (1/64 of the FP32 rate): the errors of the first float's additions, exact by TwoSum, are
+// summed in a second, and those of the second's in a third (72 bits; sums do not underflow).
+struct f3 {
+    float a, b, c;
+    __device__ __forceinline__ void add(float v) {
+        const f2 t = two_sum_f2(a, v);
+        a = t.hi;
+        add_small(t.lo);
+    }
+    // of the order of a rounding error of the sum
+    __device__ __forceinline__ void add_small(float v) {
+        const f2 t = two_sum_f2(b, v);
+        b = t.hi;
+        c = __fadd_rn(c, t.lo);
+    }
+    // the sum as hi + lo, lo below an ulp of hi or nearly so
+    __device__ __forceinline__ void value(double& hi, double& lo) const {
+        hi = (double)a + (double)b;
+        lo = ((double)a - hi) + (double)b + (double)c;   // |a| >= |b|
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
 // ----------------------------------------------------------- FP32 point solve
 // Packed residual r = R - a x + dt (K x + x K^T) with R, a, dt, K as double-float
 // and x a float vector.  R - a x is formed exactly (TwoProd); the operator term

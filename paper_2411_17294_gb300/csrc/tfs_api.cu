@@ -837,6 +837,21 @@ bool resident_path(const tfs_ctx* h) {
     return !h->is_double() && !h->classic() && !h->paper() && h->transport == 0 && h->start == TFS_START_BDF2;
 }
 
+// Steps from which one launch over them is faster than the single steps' kernels.  It reads and writes both
+// mode levels (4 words per mode value, a step moves 3), ends with one or two copies of a stress field, and holds few
+// blocks per SM where m is large; with few modes it is bound by its point solves.  Measured, single
+// against resident, us: run at 2D 512^2, 2 steps, m = 16 72 | 50, m = 48 171 | 136, m = 64 232 | 269 (3: 349 | 312);
+// 3D 128^2 x 96, m = 32, 2 steps 1237 | 1497, 3: 1870 | 1750, m = 8, 3 steps 865 | 945, 4: 1148 | 1143, m = 4,
+// 6 steps 1482 | 1534, 8: 1974 | 1938.  One step: always slower (58 | 80 at 2D 512^2, m = 32).
+int resident_run_from(const tfs_ctx* h) {
+    if (h->dim == 2) return h->m <= 48 ? 2 : 3;
+    return h->m < 8 ? 8 : (h->m < 16 ? 4 : 3);
+}
+// Reverse steps, likewise: 2D 512^2, 2 steps, m = 32 255 | 195, m = 64 393 | 397 (3: 518 | 441); 3D 128^2 x 96, 2 steps,
+// m = 8 1546 | 1490, m = 48 4245 | 3834, m = 4 1284 | 1446 (3: 1777 | 1621), m = 64 4881 | 4963 (3: 7023 | 5463).  One
+// step: 3D 128^2 x 96, m = 32 1614 | 1898.
+int resident_back_from(const tfs_ctx* h) { return h->m <= 48 && (h->dim == 2 || h->m >= 8) ? 2 : 3; }
+
 // `steps` steps with a frozen velocity gradient; sigma^{n+1} of step k goes to
 // rows + k stride (bytes).
 int run_resident(tfs_ctx* h, int steps, const void* grad_u, char* rows, size_t stride, cudaStream_t s) {
@@ -874,6 +889,19 @@ int run_resident(tfs_ctx* h, int steps, const void* grad_u, char* rows, size_t s
     h->prev_sig = older;
     h->step += steps;
     h->last_stream = s;
+    return TFS_OK;
+}
+
+// The same, one launch or step by step.
+int run_steps(tfs_ctx* h, int steps, const void* grad_u, const void* u, char* rows, size_t stride, cudaStream_t s) {
+    if (resident_path(h) && steps >= resident_run_from(h)) {
+        const int rc = step_refused(h, grad_u, u);
+        return rc != TFS_OK ? rc : run_resident(h, steps, grad_u, rows, stride, s);
+    }
+    for (int k = 0; k < steps; ++k) {
+        const int rc = do_step(h, grad_u, grad_u, u, rows + (size_t)k * stride, s);
+        if (rc != TFS_OK) return rc;
+    }
     return TFS_OK;
 }
 
@@ -1133,17 +1161,7 @@ int tfs_step(tfs_handle h, const void* grad_u_n, const void* grad_u_nm1, const v
 
 int tfs_run(tfs_handle h, int steps, const void* grad_u, const void* u, void* trajectory, void* stream) {
     if (!valid_handle(h) || steps < 1 || !trajectory || ((uintptr_t)trajectory) % 16) return TFS_ERR_ARG;
-    char* rows = (char*)trajectory;
-    const size_t stride = h->field_bytes();
-    if (resident_path(h)) {
-        const int rc = step_refused(h, grad_u, u);
-        return rc != TFS_OK ? rc : run_resident(h, steps, grad_u, rows, stride, (cudaStream_t)stream);
-    }
-    for (int k = 0; k < steps; ++k) {
-        const int rc = do_step(h, grad_u, grad_u, u, rows + (size_t)k * stride, (cudaStream_t)stream);
-        if (rc != TFS_OK) return rc;
-    }
-    return TFS_OK;
+    return run_steps(h, steps, grad_u, u, (char*)trajectory, h->field_bytes(), (cudaStream_t)stream);
 }
 
 size_t tfs_halo_bytes(tfs_handle h) {
@@ -1498,7 +1516,7 @@ static int backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* ch
     e = launch_zero(dJ_dsigma0, dfield, s);
     if (e == cudaSuccess) e = launch_zero(dJ_dgrad_u, (size_t)h->dim * h->dim * h->N * 8, s);
     if (e == cudaSuccess) e = launch_zero(L.partials, (size_t)blocks * 16, s);
-    if (resident_path(h)) {
+    if (resident_path(h) && (trajectory || K > steps ? steps : K) >= resident_back_from(h)) {
         for (int end = steps; end > 0 && e == cudaSuccess;) {
             const int start = trajectory ? 0 : (end - 1) / K * K;
             const char* rows = trajectory;
@@ -1507,8 +1525,7 @@ static int backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* ch
                 int rc = tfs_load(h, checkpoints[start / K], stream);
                 if (rc != TFS_OK) return rc;
                 if (h->step != start) return TFS_ERR_FORMAT;
-                rc = step_refused(h, grad_u, u);
-                if (rc == TFS_OK) rc = run_resident(h, end - start, grad_u, L.seg, L.seg_stride, s);
+                rc = run_steps(h, end - start, grad_u, u, L.seg, L.seg_stride, s);
                 if (rc != TFS_OK) return rc;
                 rows = L.seg;
                 stride = L.seg_stride;
@@ -1803,10 +1820,8 @@ static int backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* ch
         int rc = tfs_load(h, checkpoints[seg], stream);
         if (rc != TFS_OK) return rc;
         if (h->step != start) return TFS_ERR_FORMAT;
-        for (int n = start; n < end; ++n) {
-            rc = do_step(h, grad_u, grad_u, u, L.seg + (size_t)(n - start) * L.seg_stride, s);
-            if (rc != TFS_OK) return rc;
-        }
+        rc = run_steps(h, end - start, grad_u, u, L.seg, L.seg_stride, s);
+        if (rc != TFS_OK) return rc;
         for (int n = end - 1; n >= start; --n) {
             rc = reverse_step(n, L.seg + (size_t)(n - start) * L.seg_stride);
             if (rc != TFS_OK) return rc;

@@ -217,7 +217,8 @@ int tfs_set_state(tfs_handle h, const void* sigma0, void* stream);
    = kappa^{n-1} [d*d][N] (NULL = same as grad_u_n); u = velocity [d][N]
    (NULL allowed when transport is off); device pointers of the handle's
    element type, read only.  Enqueues the step kernel, preceded by the
-   transport pre-pass when transport is explicit (transport 2: the Krylov
+   transport pre-pass when transport is explicit (not for the stress form in FP64
+   storage, whose step kernel evaluates the stencil; transport 2: the Krylov
    solve, which synchronises `stream`).  TFS_ERR_STATE before tfs_set_state,
    TFS_ERR_NOSOE without a table, TFS_ERR_UNSTABLE when a declared velocity
    bound exceeds the explicit limit, TFS_ERR_CUDA on a failed launch. */
@@ -271,15 +272,19 @@ int tfs_get_halo(tfs_handle h, void* lo, void* hi, void* stream);
    -1) and halo_hi (the upper neighbour's first R planes: n[d-1] .. n[d-1] + R
    - 1) instead of wrapping around the slab.  Stress form with transport 0 or
    1 (TFS_ERR_ARG otherwise, and for NULL halos); other errors as tfs_step.
-   The halos are read by the transport pre-pass, on `stream`. */
+   The halos are read on `stream`, by the transport pre-pass (FP64 storage:
+   by the step kernel). */
 int tfs_step_slab(tfs_handle h, const void* grad_u_n, const void* grad_u_nm1, const void* u, const void* halo_lo,
                   const void* halo_hi, void* stream);
 
 /* Measurement hook (no counterpart in the paper): with two cudaEvent_t
    (passed as void*, both or neither), every later tfs_step records ev_before
-   on its stream just before the step kernel and ev_after just after it (the
-   transport pre-pass runs before ev_before), so that the step kernel alone
-   can be timed.  NULL, NULL turns it off.  The events are not owned. */
+   on its stream just before the step kernel and ev_after just after it, so
+   that the step kernel alone can be timed: without the transport pre-pass,
+   which runs before ev_before (the stress form in FP64 storage has none: its step
+   kernel evaluates the stencil itself).  tfs_run and the recomputed segments of
+   tfs_backward record them around each step, or around the launches that
+   take all steps at once.  NULL, NULL turns it off.  The events are not owned. */
 int tfs_set_step_events(tfs_handle h, void* ev_before, void* ev_after);
 
 /* Current step index n (number of completed steps since tfs_set_state). */

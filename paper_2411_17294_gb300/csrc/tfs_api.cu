@@ -869,13 +869,14 @@ int run_resident(tfs_ctx* h, int steps, const void* grad_u, char* rows, size_t s
     a.a = split_f2(h->eta + h->dt / h->Wi);
     a.dt = split_f2(h->dt);
     const double G = (1.0 - h->beta) / (h->Wi * h->Re);
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = h->ev_before ? cudaEventRecord(h->ev_before, s) : cudaSuccess;
     for (int k0 = 0; k0 < steps && e == cudaSuccess; k0 += kRunSteps) {
         a.steps = steps - k0 < kRunSteps ? steps - k0 : kRunSteps;
         a.rows = (float*)(rows + (size_t)k0 * stride);
         for (int k = 0; k < a.steps; ++k) a.src[k] = split_f2(h->dt * G * g_alpha(h, h->step + k0 + k));
         e = launch_resident_run(a, h->dim, h->precision == TFS_FP32, s);
     }
+    if (e == cudaSuccess && h->ev_after) e = cudaEventRecord(h->ev_after, s);
     // the stress ring as after the last step
     const int older = h->cur_sig, newest = h->prev_sig;
     if (steps >= 2 && e == cudaSuccess)

@@ -343,7 +343,8 @@ int tfs_backward(tfs_handle h, const void* dJ_dsigma_T, const void* const* check
    the state set by tfs_set_state, so that nothing is recomputed (the handle's
    forward state is left alone).  The adjoint workspace may be bound for one
    segment step.  TFS_ERR_ARG with implicit transport or the SDIRK2 start, whose reverse steps
-   need the state itself (tfs_backward). */
+   need the state itself (tfs_backward); before tfs_set_state, without a table
+   and beyond the transport's limit the errors of tfs_step. */
 int tfs_backward_run(tfs_handle h, const void* dJ_dsigma_T, const void* trajectory, int steps, const void* grad_u,
                      const void* u, double* dJ_dsigma0, double* dJ_dgrad_u, double* dJ_dWi, double* dJ_dbeta,
                      void* stream);

@@ -1847,6 +1847,8 @@ int tfs_backward_run(tfs_handle h, const void* dJ_dsigma_T, const void* trajecto
     if (!valid_handle(h) || !trajectory || ((uintptr_t)trajectory) % 16) return TFS_ERR_ARG;
     // these reverse steps solve the run's global systems again from its state
     if (h->start == TFS_START_SDIRK2 || h->implicit_transport()) return TFS_ERR_ARG;
+    const int refused = step_refused(h, grad_u, u);   // what refuses the run's steps refuses their reverse
+    if (refused != TFS_OK) return refused;
     return backward(h, dJ_dsigma_T, nullptr, 0, (const char*)trajectory, steps, grad_u, u, dJ_dsigma0, dJ_dgrad_u,
                     dJ_dWi, dJ_dbeta, stream);
 }

@@ -38,3 +38,25 @@ def test_events_are_recorded_by_a_run(precision, steps):
     assert start.elapsed_time(before) >= 0.0
     assert before.elapsed_time(after) > 0.0
     s.close()
+
+
+def test_refusals_of_the_reverse_run():
+    import torch
+    from paper_2411_17294_gb300 import tfs
+
+    def code(f):
+        with pytest.raises(tfs.TfsError) as err:
+            f()
+        return err.value.code
+
+    s, kt, _, sigma0, lam = make()
+    traj = torch.zeros((2, 3, s.N), dtype=s.dtype, device="cuda")
+    assert code(lambda: s.backward_run(lam, traj, kt)) == tfs.TFS_ERR_STATE       # no state set
+    s.close()
+    case = problem(2, (40, 24), 8, 1, False)[0]
+    s = tfs.Solver(2, (40, 24), 0.5, 1.3, 0.4, 2e-3, m=8, precision=1, transport=False)
+    s.set_state(sigma0)
+    assert code(lambda: s.backward_run(lam, traj, kt)) == tfs.TFS_ERR_NOSOE       # no table
+    s.set_soe(case["mu"], case["w"])
+    s.backward_run(lam, s.run(2, kt), kt)
+    s.close()

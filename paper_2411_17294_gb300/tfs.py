@@ -246,11 +246,12 @@ class Solver:
 
     def run(self, steps: int, grad_u, u=None, stream=None):
         """`steps` steps with the frozen grad_u (tfs_run); returns the stress
-        after each step, [steps, nc, N].  Tensors as for step()."""
+        after each step, [steps, nc, N], a tensor of `stream` (another stream that
+        reads it waits for the run, as for any tensor of a stream).  Tensors as for step()."""
         torch = _torch()
-        traj = torch.empty((int(steps), self.nc, self.N), dtype=self.dtype, device=self.device)
-        if stream is not None:
-            traj.record_stream(stream)
+        # allocated for the stream that writes it: a block freed on the current stream may have work pending there
+        with torch.cuda.stream(stream):
+            traj = torch.empty((int(steps), self.nc, self.N), dtype=self.dtype, device=self.device)
         check(self.lib.tfs_run(self.h, int(steps), ctypes.c_void_p(grad_u.data_ptr()),
                                ctypes.c_void_p(u.data_ptr() if u is not None else 0),
                                ctypes.c_void_p(traj.data_ptr()),

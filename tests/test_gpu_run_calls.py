@@ -60,3 +60,22 @@ def test_refusals_of_the_reverse_run():
     s.set_soe(case["mu"], case["w"])
     s.backward_run(lam, s.run(2, kt), kt)
     s.close()
+
+
+def test_trajectory_of_another_stream():
+    # a block of the trajectory's size, freed on the current stream with a write to it still pending there
+    import torch
+    s, kt, _, sigma0, _ = make()
+    s.set_state(sigma0)
+    ref = s.run(40, kt)
+    s.set_state(sigma0)
+    side = torch.cuda.Stream()
+    block = torch.empty_like(ref)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(50000000)
+    block.fill_(7.0)
+    del block
+    got = s.run(40, kt, stream=side)
+    torch.cuda.synchronize()
+    assert torch.equal(got, ref)
+    s.close()

@@ -51,12 +51,13 @@ struct PackedIndex {
     }
 };
 
-// The point system M = a I - scale L(K) by FP64 Gaussian elimination: component c of
-// M^-1 R.  Returns false when a pivot vanishes.
-template <int DIM>
-__device__ __noinline__ bool solve_by_elimination(const double* sK, const double* sR, double a, double scale, int c,
-                                                   bool transposed, double* out) {
+// The point system M = a I - scale L(K) (scale 1 where none is given: a further argument spills in the 3D
+// step) by FP64 Gaussian elimination: component c of M^-1 R.  Returns false when a pivot vanishes.
+template <int DIM, bool TRANSPOSED, typename... Scale>
+__device__ __noinline__ bool solve_by_elimination(const double* sK, const double* sR, double a, int c, double* out,
+                                                   Scale... given) {
     constexpr int NC = Packed<DIM>::NC;
+    const double scale = (1.0 * ... * given);
     double K[3][3], x[NC], M[NC][NC];
 #pragma unroll
     for (int i = 0; i < DIM; ++i)
@@ -65,7 +66,7 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 #pragma unroll
     for (int r = 0; r < NC; ++r) x[r] = sR[r * kT64];
     assemble_M<DIM>(K, a, scale, M);
-    if (transposed) {
+    if (TRANSPOSED) {
 #pragma unroll
         for (int i = 0; i < NC; ++i)
 #pragma unroll
@@ -94,7 +95,7 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 // y2 is |y2| q: q < 2^-18 leaves it below the last bit, and then |y2| is below 2^-36 |x|;
 // otherwise further passes follow.  FP64 elimination with partial pivoting takes over where
 // the refinement does not contract, where a right-hand side or solution is outside the FP32
-// images' range, where the matrix is (its entries' sum from 2^64 up: what a y below the FP32
+// images' range, where the matrix is (its entries' sum, or its dominant diagonal's, from 2^64 up: what a y below the FP32
 // normal numbers contributes to a residual is then not negligible any more, and from 2^128 the
 // factors are not finite), and for a component whose own residual is so far below the point's
 // others (2^-126) that its image or its y vanishes.
@@ -119,21 +120,30 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             F.a[ro][k] = v;
         });
     });
+    // the entries' magnitude: of a dominant matrix the diagonal bounds all
+    const bool dominant = row_dominant<NC>(F);
     float entries = 0.0f;
     static_for<0, NC>([&](auto rr) {
         constexpr int ro = decltype(rr)::value;
-        float off = 0.0f;   // as row_dominant() forms it
-        static_for<0, NC>([&](auto kk) {
-            constexpr int k = decltype(kk)::value;
-            if (k != ro) off += fabsf(F.a[ro][k]);
-        });
-        entries += off + fabsf(F.a[ro][ro]);
+        entries += fabsf(F.a[ro][ro]);
     });
-    bool good = row_dominant<NC>(F) ? lu32_factor_nopivot<NC>(F, 1e-30f) : lu32_factor<NC>(F, 1e-30f);
-    good = good && entries < 18446744073709551616.0f;   // false for a NaN
+    bool good;
+    if (dominant) {
+        good = lu32_factor_nopivot<NC>(F, 1e-30f);
+    } else {
+        static_for<0, NC>([&](auto rr) {
+            constexpr int ro = decltype(rr)::value;
+            static_for<0, NC>([&](auto kk) {
+                constexpr int k = decltype(kk)::value;
+                if (k != ro) entries += fabsf(F.a[ro][k]);
+            });
+        });
+        good = lu32_factor<NC>(F, 1e-30f);
+    }
+    good = good && entries < 18446744073709551616.0f;   // 2^64; false for a NaN
     int e0 = 0;
     constexpr int kMaxPass = 8;
-    bool done = false, lost = false;
+    bool done = false;
     double x = 0.0;
     for (int pass = 0; pass < kMaxPass; ++pass) {
         const double* rb = pass == 0 ? sR : sR + (1 + (pass & 1)) * NC * kT64;
@@ -153,11 +163,6 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             y[k] = scaled_float(rv[k], emax);
         }
         if (pass == 0) good = good && emax < 0x7ff && (emax > 200 || zero);
-        float own = 0.0f;
-        static_for<0, NC>([&](auto kk) {
-            constexpr int k = decltype(kk)::value;
-            if (c == k) own = y[k];
-        });
         lu32_solve<NC>(F, y);
         unsigned ymax = 0u;
 #pragma unroll
@@ -173,7 +178,9 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             // a point's passes are its own, whatever the other points of its tile still need
             if (c == k && !done) {
                 x += unscaled_double(y[k], emax);
-                lost = lost || (!zero64(r) && (own == 0.0f || (__float_as_uint(y[k]) & 0x7fffffffu) < 0x00800000u));
+                // lost in scaling: marked for elimination (nothing else makes x a NaN from finite numbers)
+                if (!zero64(r) && (biased_exp(r) <= emax - 127 || (__float_as_uint(y[k]) & 0x7fffffffu) < 0x00800000u))
+                    x = __hiloint2double(0x7ff80000, 0);
             }
         });
         done = done || zero || (pass >= 2 && small);
@@ -206,7 +213,10 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
         named_sync<NC * 32>();
     }
     bool ok = true;
-    if (!good || !done || lost) ok = solve_by_elimination<DIM>(sK, sR, a, scale, c, TRANSPOSED, &x);
+    if (!good || !done || !finite64(x)) {
+        if constexpr (SCALED) ok = solve_by_elimination<DIM, TRANSPOSED>(sK, sR, a, c, &x, scale);
+        else ok = solve_by_elimination<DIM, TRANSPOSED>(sK, sR, a, c, &x);
+    }
     *out = x;
     return ok;
 }

@@ -34,6 +34,8 @@
 // at 3D 160^3, 7.3e-16 against 8.9e-16 at 2D 1024^2).
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "tfs_device.cuh"
 #include "tfs_internal.h"
 #include "tfs_solve64.cuh"
@@ -63,7 +65,13 @@ __host__ __device__ constexpr size_t smem64_bytes(int m, int groups) {
 
 // Products of the step's scalars, formed once on the host.
 struct Step64 {
-    double src;        // G g (kappa* comes with dt)
+    // what kappa* is scaled by: dt, in the paper's variable dt xi with xi's power of two apart (xi = frac 2^kexp,
+    // frac in [1, 2), so that xi = 0, a table without weight, divides nothing; then kexp is far out of range)
+    double scale;
+    double src;        // dt G g / scale
+    double inv_frac;   // 1 / frac
+    double pow2;       // 2^kexp, or 0
+    int kexp;
     double g6[3];      // dt / (6 h_a)
     double lap[3];     // eps dt / h_a^2
     float inv_h[3];
@@ -171,7 +179,7 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
     double* sQ = sm64;                          // Q'_j [m][NC][32]
     double* sH = sQ + (size_t)m * NC * kT64;    // partial history sums [G][NC][32]
     double* sR = sH + G * NC * kT64;            // right-hand side, then two buffers of residuals [3][NC][32]
-    double* sK = sR + 3 * NC * kT64;            // dt kappa* [DD][32]
+    double* sK = sR + 3 * NC * kT64;            // dt kappa* (the paper's variable: dt frac kappa*) [DD][32]
     double* sC = sK + DD * kT64;                // stencil coefficients
     // dt kappa* in FP32 (the paper's variable: dt xi kappa*, the operator's)
     float* sKf = reinterpret_cast<float*>(sC + Shape64<DIM>::kCoef * kT64);
@@ -184,9 +192,9 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
     // ---- velocity gradient entries and stencil coefficients, spread over the warps
     for (int k = w; k < DD; k += NC * G) {
         const long long q = (long long)k * A.N + pc;
-        const double v = A.dt * fma(2.0, A.kap_n[q], -A.kap_nm1[q]);
+        const double v = B.scale * fma(2.0, A.kap_n[q], -A.kap_nm1[q]);
         sK[k * kT64 + lane] = v;
-        sKf[k * kT64 + lane] = (float)(PAPER ? A.xi * v : v);
+        sKf[k * kT64 + lane] = PAPER ? (float)v * (float)B.pow2 : (float)v;
     }
     if (TR == kInStep && w == NC * G - 1) {
         double u[DIM];
@@ -269,7 +277,7 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
             for (int l = 0; l < DIM; ++l)
                 lh = fma(sK[(ci * DIM + l) * kT64 + lane], hat(l, cj),
                          fma(hat(ci, l), sK[(cj * DIM + l) * kT64 + lane], lh));
-            r = fma(2.0, A.sig_n[q], -0.5 * A.sig_nm1[q]) - A.dt * A.inv_wi * H + fma(B.src, ks, lh);
+            r = fma(2.0, A.sig_n[q], -0.5 * A.sig_nm1[q]) - A.dt * A.inv_wi * H + fma(B.src, ks, B.inv_frac * lh);
             if (TR == kFromPrepass) r -= A.trans[q];
         } else {
             s0 = has_s0 ? A.sigma0[q] : 0.0;
@@ -281,7 +289,7 @@ __global__ void __launch_bounds__(kT64* Packed<DIM>::NC* G, G > 1 ? 1 : (DIM == 
     __syncthreads();
     if (grp == 0) {
         unsigned fl = 0u;
-        if (!refine_solve64<DIM, false, PAPER>(sK + lane, sKf + lane, sR + lane, A.a, B.a, c, r, &x, PAPER ? A.xi : 1.0) &&
+        if (!refine_solve64<DIM, false, PAPER>(sK + lane, sKf + lane, sR + lane, A.a, B.a, c, r, &x, B.pow2, B.kexp) &&
             active)
             fl |= 2u;
         const long long q = (long long)c * A.N + p;
@@ -337,7 +345,14 @@ cudaError_t launch64(const FwdArgs<double>& a, const LaunchCfg& cfg, long long t
     if (e != cudaSuccess) return e;
     const size_t dyn = smem64_bytes<DIM>(cfg.classic ? 0 : a.m, G);
     Step64 b;
-    b.src = a.G * a.g;
+    const bool has = !PAPER || (a.xi > 0.0 && std::isfinite(a.xi));
+    const int kexp = PAPER && has ? std::ilogb(a.xi) : 0;
+    const double frac = PAPER && has ? std::ldexp(a.xi, -kexp) : 1.0;
+    b.scale = a.dt * frac;
+    b.src = a.G * a.g / frac;
+    b.inv_frac = 1.0 / frac;
+    b.pow2 = has ? std::ldexp(1.0, kexp) : 0.0;
+    b.kexp = has ? kexp : -10000;
     for (int i = 0; i < 3; ++i) {
         b.g6[i] = a.dt * a.inv_h[i] / 6.0;
         b.lap[i] = a.eps * a.dt * a.inv_h[i] * a.inv_h[i];

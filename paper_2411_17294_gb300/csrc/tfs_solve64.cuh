@@ -86,7 +86,7 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 
 // Component c of M^-1 R (TRANSPOSED: M^-T R), M = a I - scale L(K), for this lane's point; every
 // lane of the NC warps of the tile calls it.  sK: K in FP64 [d*d][32]; sKf: scale K in FP32
-// (SCALED false: scale is 1); sR: R [NC][32] followed by two buffers of that size for the residuals (all at this
+// (SCALED false: scale is 1; else a power of two 2^kexp, or 0 with kexp far below the exponents' range); sR: R [NC][32] followed by two buffers of that size for the residuals (all at this
 // lane); r: this thread's entry of R.  Returns false when a pivot vanishes.
 //
 // The warps factor the tile's 32 matrices in FP32, each for itself (the FP32 pipe is idle),
@@ -101,8 +101,7 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 // others (2^-126) that its image or its y vanishes.
 template <int DIM, bool TRANSPOSED, bool SCALED = false>
 __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sKf, double* sR, double a, float af,
-                                               int c, double r, double* out, double scale = 1.0) {
-    static_assert(!(TRANSPOSED && SCALED), "the transposed systems take K scaled");
+                                               int c, double r, double* out, double scale = 1.0, int kexp = 0) {
     constexpr int NC = Packed<DIM>::NC;
     LU32<NC> F;
     static_for<0, NC>([&](auto rr) {
@@ -169,7 +168,7 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
         for (int k = 0; k < NC; ++k) ymax = max(ymax, __float_as_uint(y[k]) & 0x7fffffffu);
         const int ey = (int)(ymax >> 23) + emax;       // exponent of the correction (biased by 127 + 1023)
         if (pass == 0) {
-            good = good && ymax < 0x7f800000u && ey - 127 < 0x7ff;
+            good = good && ymax < 0x7f800000u && ey - 127 + (SCALED ? max(kexp, 0) : 0) < 0x7ff;
             e0 = ey;
         }
         const bool small = ymax != 0u && ey <= e0 - 36;
@@ -191,22 +190,21 @@ __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sK
             if (c == k) {
                 constexpr int i = Packed<DIM>::I(k), j = Packed<DIM>::J(k);
                 r = fma(-a, unscaled_double(y[k], emax), r);
-                double q = SCALED ? 0.0 : r;
+                const int ek = SCALED ? emax + kexp : emax;   // y scale
                 static_for<0, DIM>([&](auto ll) {
                     constexpr int l = decltype(ll)::value;
                     constexpr int lj = PackedIndex<DIM>::at(l, j), li = PackedIndex<DIM>::at(l, i);
                     if constexpr (!TRANSPOSED) {
-                        q = fma(sK[(i * DIM + l) * kT64], unscaled_double(y[lj], emax), q);
-                        q = fma(sK[(j * DIM + l) * kT64], unscaled_double(y[li], emax), q);
+                        r = fma(sK[(i * DIM + l) * kT64], unscaled_double(y[lj], ek), r);
+                        r = fma(sK[(j * DIM + l) * kT64], unscaled_double(y[li], ek), r);
                     } else {
                         // (L^T y)_ij = sum_l K_li Y_lj + K_lj Y_li (once for i = j), Y symmetric
                         // with the diagonal doubled
-                        q = fma(sK[(l * DIM + i) * kT64], unscaled_double(l == j ? 2.0f * y[lj] : y[lj], emax), q);
+                        r = fma(sK[(l * DIM + i) * kT64], unscaled_double(l == j ? 2.0f * y[lj] : y[lj], ek), r);
                         if constexpr (i != j)
-                            q = fma(sK[(l * DIM + j) * kT64], unscaled_double(l == i ? 2.0f * y[li] : y[li], emax), q);
+                            r = fma(sK[(l * DIM + j) * kT64], unscaled_double(l == i ? 2.0f * y[li] : y[li], ek), r);
                     }
                 });
-                r = SCALED ? fma(scale, q, r) : q;
             }
         });
         sR[(1 + ((pass + 1) & 1)) * NC * kT64 + c * kT64] = r;

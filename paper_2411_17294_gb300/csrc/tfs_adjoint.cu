@@ -411,15 +411,17 @@ struct F3c {
 };
 struct GatherScales {
     double g6[3], lap[3];           // dt / (6 h_a), eps dt / h_a^2
-    F3c tap[3][4], lapf[3][2];      // g6 times 1, 2, 3, 6 and lap times 1, -2, times 1/unscale
+    F3c tap[3][7], lapf[3][2];      // g6 times 1, 2, 3, 6 (by that index) and lap times 1, -2, times 1/unscale
     double unscale;                 // a power of two
 };
 
-// six times the weight of tap k, 0 where the stencil does not read it
-__device__ __forceinline__ float tap_weight(int stencil, bool forward_u, int k) {
-    if (stencil == 1) return k == 1 ? 3.0f : (k == -1 ? -3.0f : 0.0f);
-    if (forward_u) return k == -2 ? 1.0f : (k == -1 ? -6.0f : (k == 0 ? 3.0f : (k == 1 ? 2.0f : 0.0f)));
-    return k == -1 ? -2.0f : (k == 0 ? -3.0f : (k == 1 ? 6.0f : (k == 2 ? -1.0f : 0.0f)));
+// Six times the weight of tap k: `forward` where u >= 0 (the upwind stencil's side), 0 where the stencil
+// does not read it.
+template <int STENCIL>
+__host__ __device__ constexpr int tap_weight(bool forward, int k) {
+    if (STENCIL == 1) return 3 * ((k == 1) - (k == -1));
+    return forward ? (k == -2) - 6 * (k == -1) + 3 * (k == 0) + 2 * (k == 1)
+                   : -2 * (k == -1) - 3 * (k == 0) + 6 * (k == 1) - (k == 2);
 }
 
 // Offset of the periodic neighbour off (|off| <= 2) points away along an axis of n points at v.
@@ -435,11 +437,10 @@ __device__ __forceinline__ long long neighbour(int v, int off, int n, long long 
 __device__ __forceinline__ bool is_zero(float v) { return v == 0.0f; }
 __device__ __forceinline__ bool is_zero(double v) { return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0; }
 
-// Calls tap(offset of p, axis, k, u_a(p), six times the tap's weight, whether the Laplacian reads it) for every
-// point p whose stencil reads q.
-template <int DIM, typename TU, typename F>
-__device__ __forceinline__ void for_taps(const AdjArgs<double>& A, const TU* __restrict__ u, int stencil, long long q,
-                                         F&& tap) {
+// Calls tap(offset of p, axis, k, u_a(p), whether u_a(p) >= 0, whether the Laplacian reads q) for every point p
+// whose stencil reads q.
+template <int DIM, int STENCIL, typename TU, typename F>
+__device__ __forceinline__ void for_taps(const AdjArgs<double>& A, const TU* __restrict__ u, long long q, F&& tap) {
     const unsigned qu = (unsigned)q, r1 = qu / (unsigned)A.n0;
     const int co[3] = {(int)(qu % (unsigned)A.n0), (int)(DIM == 3 ? r1 % (unsigned)A.n1 : r1),
                        (int)(DIM == 3 ? r1 / (unsigned)A.n1 : 0)};
@@ -450,35 +451,41 @@ __device__ __forceinline__ void for_taps(const AdjArgs<double>& A, const TU* __r
         constexpr int ax = decltype(aa)::value;
         static_for<0, 5>([&](auto kk) {
             constexpr int k = decltype(kk)::value - 2;
-            const long long p = q + neighbour(co[ax], -k, nn[ax], st[ax]);
-            const TU ua = __ldg(u + (long long)ax * A.N + p);
-            const float w6 = tap_weight(stencil, ua >= (TU)0, k);
-            const bool lap = diffusion && k >= -1 && k <= 1;
-            if ((w6 != 0.0f && !is_zero(ua)) || lap) tap(p, aa, std::integral_constant<int, k>{}, ua, w6, lap);
+            constexpr int wf = tap_weight<STENCIL>(true, k), wb = tap_weight<STENCIL>(false, k);
+            constexpr bool near = k >= -1 && k <= 1;
+            if constexpr (wf != 0 || wb != 0 || near) {
+                const bool lap = near && diffusion;
+                const long long p = q + neighbour(co[ax], -k, nn[ax], st[ax]);
+                const TU ua = __ldg(u + (long long)ax * A.N + p);
+                const bool forward = ua >= (TU)0;
+                if ((!is_zero(ua) && (forward ? wf : wb) != 0) || lap)
+                    tap(p, aa, std::integral_constant<int, k>{}, ua, forward, lap);
+            }
         });
     });
 }
 
 // lamE(q) in FP64: two operations per tap shared by the components and one FMA per component.
-template <int DIM, typename TU>
+template <int DIM, int STENCIL, typename TU>
 __device__ __forceinline__ void gather(const AdjArgs<double>& A, const GatherScales& Q, const TU* __restrict__ lamR,
-                                       const TU* __restrict__ u, int stencil, long long q, double* lamE) {
+                                       const TU* __restrict__ u, long long q, double* lamE) {
     constexpr int NC = Packed<DIM>::NC;
 #pragma unroll
     for (int c = 0; c < NC; ++c) lamE[c] = 0.0;
-    for_taps<DIM>(A, u, stencil, q, [&](long long p, auto aa, auto kk, TU ua, float w6, bool lap) {
+    for_taps<DIM, STENCIL>(A, u, q, [&](long long p, auto aa, auto kk, TU ua, bool forward, bool lap) {
         constexpr int ax = decltype(aa)::value, k = decltype(kk)::value;
-        double w = Q.g6[ax] * (double)ua * (double)-w6;
+        constexpr double wf = -tap_weight<STENCIL>(true, k), wb = -tap_weight<STENCIL>(false, k);
+        double w = Q.g6[ax] * (double)ua * (forward ? wf : wb);
         if (lap) w = fma(k == 0 ? -2.0 : 1.0, Q.lap[ax], w);
 #pragma unroll
         for (int c = 0; c < NC; ++c) lamE[c] = fma(w, (double)__ldg(lamR + (long long)c * A.N + p), lamE[c]);
     });
 }
 
-template <int DIM>
+template <int DIM, int STENCIL>
 __device__ __noinline__ void gather_out_of_range(const AdjArgs<double>& A, const GatherScales& Q, const float* lamR,
-                                                 const float* u, int stencil, long long q, double* lamE) {
-    gather<DIM, float>(A, Q, lamR, u, stencil, q, lamE);
+                                                 const float* u, long long q, double* lamE) {
+    gather<DIM, STENCIL, float>(A, Q, lamR, u, q, lamE);
 }
 
 // FP64 storage: all in FP64.  FP32 storage (lamR and u hold floats): the FP64 pipe's rate, 1/64 of the FP32
@@ -487,30 +494,34 @@ __device__ __noinline__ void gather_out_of_range(const AdjArgs<double>& A, const
 // of its products' magnitudes, 1.1e-16 against 4.3e-16; two floats 2.7e-14).  The weights carry a power of two that
 // keeps the products' rounding errors representable for every normal lamR; sums beyond
 // the float range are formed again in FP64.  Thread = point; the x rows of
-// neighbouring threads come from L1.  3D 64^3, FP32 storage: 61 us, against 92 in FP64 with conversions by integer
+// neighbouring threads come from L1.  3D 64^3, FP32 storage: 60 us, against 92 in FP64 with conversions by integer
 // operations, 140 with the FP64 pipe's, and 33 for sums of two floats.
-template <typename TU, int DIM>
+template <typename TU, int DIM, int STENCIL>
 __global__ void __launch_bounds__(128) adj_transport_kernel(const AdjArgs<double> A, const GatherScales Q,
-                                                            const TU* __restrict__ lamR, const TU* __restrict__ u,
-                                                            const int stencil) {
+                                                            const TU* __restrict__ lamR, const TU* __restrict__ u) {
     constexpr int NC = Packed<DIM>::NC;
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= A.N) return;
     double lamE[NC];
     if constexpr (sizeof(TU) == 8) {
-        gather<DIM, TU>(A, Q, lamR, u, stencil, q, lamE);
+        gather<DIM, STENCIL, TU>(A, Q, lamR, u, q, lamE);
     } else {
         f3 s[NC];
 #pragma unroll
         for (int c = 0; c < NC; ++c) s[c] = f3{0.0f, 0.0f, 0.0f};
-        for_taps<DIM>(A, u, stencil, q, [&](long long p, auto aa, auto kk, float ua, float w6, bool lap) {
+        for_taps<DIM, STENCIL>(A, u, q, [&](long long p, auto aa, auto kk, float ua, bool forward, bool lap) {
             constexpr int ax = decltype(aa)::value, k = decltype(kk)::value;
+            constexpr int wf = tap_weight<STENCIL>(true, k), wb = tap_weight<STENCIL>(false, k);
             // -w6 g6 u [+ lap] as three floats
-            const float m = fabsf(w6), us = m == 0.0f ? 0.0f : (w6 > 0.0f ? -ua : ua);
-            const F3c g = m == 1.0f ? Q.tap[ax][0] : (m == 2.0f ? Q.tap[ax][1] : (m == 3.0f ? Q.tap[ax][2] : Q.tap[ax][3]));
-            const f2 p0 = two_prod(g.a, us), p1 = two_prod(g.b, us);
-            const f2 t = two_sum_f2(p0.lo, p1.hi), h = fast_two_sum(p0.hi, t.hi);
-            f3 w{h.hi, h.lo, __fadd_rn(t.lo, __fmaf_rn(g.c, us, p1.lo))};
+            f3 w{0.0f, 0.0f, 0.0f};
+            if constexpr (wf != 0 || wb != 0) {
+                constexpr int mf = wf < 0 ? -wf : wf, mb = wb < 0 ? -wb : wb;
+                const F3c g = (forward ? mf : mb) == mf ? Q.tap[ax][mf] : Q.tap[ax][mb];
+                const float us = (forward ? wf : wb) > 0 ? -ua : ua;
+                const f2 p0 = two_prod(g.a, us), p1 = two_prod(g.b, us);
+                const f2 t = two_sum_f2(p0.lo, p1.hi), h = fast_two_sum(p0.hi, t.hi);
+                w = f3{h.hi, h.lo, __fadd_rn(t.lo, __fmaf_rn(g.c, us, p1.lo))};
+            }
             if (lap) {
                 const F3c l = Q.lapf[ax][k == 0 ? 1 : 0];
                 w.add(l.a);
@@ -535,7 +546,7 @@ __global__ void __launch_bounds__(128) adj_transport_kernel(const AdjArgs<double
         }
         if (!finite) {
             double out[NC];
-            gather_out_of_range<DIM>(A, Q, lamR, u, stencil, q, out);
+            gather_out_of_range<DIM, STENCIL>(A, Q, lamR, u, q, out);
 #pragma unroll
             for (int c = 0; c < NC; ++c) lamE[c] = out[c];
         }
@@ -617,22 +628,23 @@ cudaError_t launch_adjoint_transport(const AdjArgs<double>& a, const void* lamR,
         if (i < cfg.dim) top = std::fmax(top, std::fmax(q.g6[i], q.lap[i]));
     }
     const int up = top > 0.0 && std::isfinite(top) ? 30 - std::ilogb(top) : 0;   // weights of unit velocity near 2^30
-    const double factor[4] = {1.0, 2.0, 3.0, 6.0};
     for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 4; ++j) q.tap[i][j] = split_f3(std::ldexp(factor[j] * q.g6[i], up));
+        for (int j = 0; j < 7; ++j) q.tap[i][j] = split_f3(std::ldexp(j * q.g6[i], up));
         for (int j = 0; j < 2; ++j) q.lapf[i][j] = split_f3(std::ldexp((j ? -2.0 : 1.0) * q.lap[i], up));
     }
     q.unscale = std::ldexp(1.0, -up);
+    auto launch = [&](auto type, auto dim) {
+        using TU = decltype(type);
+        constexpr int D = decltype(dim)::value;
+        auto kernel = cfg.stencil == 1 ? adj_transport_kernel<TU, D, 1> : adj_transport_kernel<TU, D, 0>;
+        kernel<<<blocks, threads, 0, s>>>(a, q, (const TU*)lamR, (const TU*)u);
+    };
     if (cfg.dim == 2) {
-        if (is_double)
-            adj_transport_kernel<double, 2><<<blocks, threads, 0, s>>>(a, q, (const double*)lamR, (const double*)u, cfg.stencil);
-        else
-            adj_transport_kernel<float, 2><<<blocks, threads, 0, s>>>(a, q, (const float*)lamR, (const float*)u, cfg.stencil);
+        if (is_double) launch(0.0, std::integral_constant<int, 2>{});
+        else launch(0.0f, std::integral_constant<int, 2>{});
     } else {
-        if (is_double)
-            adj_transport_kernel<double, 3><<<blocks, threads, 0, s>>>(a, q, (const double*)lamR, (const double*)u, cfg.stencil);
-        else
-            adj_transport_kernel<float, 3><<<blocks, threads, 0, s>>>(a, q, (const float*)lamR, (const float*)u, cfg.stencil);
+        if (is_double) launch(0.0, std::integral_constant<int, 3>{});
+        else launch(0.0f, std::integral_constant<int, 3>{});
     }
     return cudaGetLastError();
 }

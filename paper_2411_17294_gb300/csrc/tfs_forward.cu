@@ -1204,7 +1204,11 @@ cudaError_t launch_prepass(const FwdArgs<T>& ta, const LaunchCfg& cfg, cudaStrea
     } else {
         const int threads = 256;
         long long blocks = (ta.N + threads - 1) / threads;
-        if (blocks > 152ll * 16) blocks = 152ll * 16;
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if (blocks > sms * 16ll) blocks = sms * 16ll;
         transport_kernel<T, DIM><<<(unsigned)blocks, threads, 0, s>>>(ta, cfg.stencil);
     }
     return cudaGetLastError();

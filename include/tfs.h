@@ -237,8 +237,8 @@ int tfs_get_stress(tfs_handle h, void* out, void* stream);
    aligned) receives the stress after each step (Psi with TFS_FORM_PAPER), and
    the state is that after the last.  The FP32 stress form with alpha < 1, BDF2
    start and transport 0 keeps its modes in registers over the steps (bitwise
-   the same stresses) from the number of steps on at which that is faster.  Enqueues on `stream` (implicit transport synchronises);
-   errors as tfs_step, TFS_ERR_ARG for steps < 1 or a NULL or misaligned
+   the same stresses) from the number of steps on at which that is faster.
+   Enqueues on `stream` (implicit transport synchronises); errors as tfs_step, TFS_ERR_ARG for steps < 1 or a NULL or misaligned
    trajectory. */
 int tfs_run(tfs_handle h, int steps, const void* grad_u, const void* u, void* trajectory, void* stream);
 

@@ -435,7 +435,9 @@ __device__ __forceinline__ long long neighbour(int v, int off, int n, long long 
 }
 
 __device__ __forceinline__ bool is_zero(float v) { return v == 0.0f; }
-__device__ __forceinline__ bool is_zero(double v) { return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0; }
+__device__ __forceinline__ bool is_zero(double v) {
+    return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0;
+}
 
 // Calls tap(offset of p, axis, k, u_a(p), whether u_a(p) >= 0, whether the Laplacian reads q) for every point p
 // whose stencil reads q.

@@ -847,8 +847,8 @@ int resident_run_from(const tfs_ctx* h) {
     if (h->dim == 2) return h->m <= 48 ? 2 : 3;
     return h->m < 8 ? 8 : (h->m < 16 ? 4 : 3);
 }
-// Reverse steps, likewise: 2D 512^2, 2 steps, m = 32 255 | 195, m = 64 393 | 397 (3: 518 | 441); 3D 128^2 x 96, 2 steps,
-// m = 8 1546 | 1490, m = 48 4245 | 3834, m = 4 1284 | 1446 (3: 1777 | 1621), m = 64 4881 | 4963 (3: 7023 | 5463).  One
+// Reverse steps, likewise: 2D 512^2, 2 steps, m = 32 255 | 195, m = 64 393 | 397 (3: 518 | 441); 3D 128^2 x 96,
+// 2 steps, m = 8 1546 | 1490, m = 48 4245 | 3834, m = 4 1284 | 1446 (3: 1777 | 1621), m = 64 4881 | 4963 (3: 7023 | 5463).  One
 // step: 3D 128^2 x 96, m = 32 1614 | 1898.
 int resident_back_from(const tfs_ctx* h) { return h->m <= 48 && (h->dim == 2 || h->m >= 8) ? 2 : 3; }
 

@@ -86,8 +86,9 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 
 // Component c of M^-1 R (TRANSPOSED: M^-T R), M = a I - scale L(K), for this lane's point; every
 // lane of the NC warps of the tile calls it.  sK: K in FP64 [d*d][32]; sKf: scale K in FP32
-// (SCALED false: scale is 1; else a power of two 2^kexp, or 0 with kexp far below the exponents' range); sR: R [NC][32] followed by two buffers of that size for the residuals (all at this
-// lane); r: this thread's entry of R.  Returns false when a pivot vanishes.
+// (SCALED false: scale is 1; else a power of two 2^kexp, or 0 with kexp far below the
+// exponents' range); sR: R [NC][32] followed by two buffers of that size for the residuals (all
+// at this lane); r: this thread's entry of R.  Returns false when a pivot vanishes.
 //
 // The warps factor the tile's 32 matrices in FP32, each for itself (the FP32 pipe is idle),
 // and x = y0 + y1 + ..., each y the FP32 solution for the residual so far, each thread
@@ -95,9 +96,9 @@ __device__ __noinline__ bool solve_by_elimination(const double* sK, const double
 // y2 is |y2| q: q < 2^-18 leaves it below the last bit, and then |y2| is below 2^-36 |x|;
 // otherwise further passes follow.  FP64 elimination with partial pivoting takes over where
 // the refinement does not contract, where a right-hand side or solution is outside the FP32
-// images' range, where the matrix is (its entries' sum, or its dominant diagonal's, from 2^64 up: what a y below the FP32
-// normal numbers contributes to a residual is then not negligible any more, and from 2^128 the
-// factors are not finite), and for a component whose own residual is so far below the point's
+// images' range, where the matrix is (its entries' sum, or its dominant diagonal's, from 2^64 up:
+// what a y below the FP32 normal numbers contributes to a residual is then not negligible any
+// more, and from 2^128 the factors are not finite), and for a component whose own residual is so far below the point's
 // others (2^-126) that its image or its y vanishes.
 template <int DIM, bool TRANSPOSED, bool SCALED = false>
 __device__ __forceinline__ bool refine_solve64(const double* sK, const float* sKf, double* sR, double a, float af,

@@ -290,8 +290,8 @@ class Solver:
 
     def set_step_events(self, ev_before, ev_after):
         """Record torch.cuda.Event objects around the step kernel of each later
-        step, or around the launches with which run() takes all steps at once (None, None turns it off).  torch creates an event's handle on its
-        first record, so each event must have been recorded once before."""
+        step, or around the launches with which run() takes all steps at once
+        (None, None turns it off).  torch creates an event's handle on its first record, so each event must have been recorded once before."""
         def handle(ev):
             if ev is None:
                 return 0

@@ -1,5 +1,6 @@
 """The paper's variable with a table whose weights are all zero (accepted by
-tfs_set_soe): Psi = xi Phi + h = 0 at every step, in both storage forms; Phi follows its own equation without dividing by xi = 0."""
+tfs_set_soe): Psi = xi Phi + h = 0 at every step, in both storage forms; Phi
+follows its own equation without dividing by xi = 0."""
 import numpy as np
 import pytest
 

@@ -440,8 +440,8 @@ __device__ __forceinline__ bool is_zero(double v) {
 }
 
 // Calls tap(offset of p, axis, k, u_a(p), whether u_a(p) >= 0, whether the Laplacian reads q) for every point p
-// whose stencil reads q.
-template <int DIM, int STENCIL, typename TU, typename F>
+// whose stencil reads q (CENTRE: q itself too).
+template <int DIM, int STENCIL, bool CENTRE, typename TU, typename F>
 __device__ __forceinline__ void for_taps(const AdjArgs<double>& A, const TU* __restrict__ u, long long q, F&& tap) {
     const unsigned qu = (unsigned)q, r1 = qu / (unsigned)A.n0;
     const int co[3] = {(int)(qu % (unsigned)A.n0), (int)(DIM == 3 ? r1 % (unsigned)A.n1 : r1),
@@ -455,7 +455,7 @@ __device__ __forceinline__ void for_taps(const AdjArgs<double>& A, const TU* __r
             constexpr int k = decltype(kk)::value - 2;
             constexpr int wf = tap_weight<STENCIL>(true, k), wb = tap_weight<STENCIL>(false, k);
             constexpr bool near = k >= -1 && k <= 1;
-            if constexpr (wf != 0 || wb != 0 || near) {
+            if constexpr ((wf != 0 || wb != 0 || near) && (CENTRE || k != 0)) {
                 const bool lap = near && diffusion;
                 const long long p = q + neighbour(co[ax], -k, nn[ax], st[ax]);
                 const TU ua = __ldg(u + (long long)ax * A.N + p);
@@ -474,7 +474,7 @@ __device__ __forceinline__ void gather(const AdjArgs<double>& A, const GatherSca
     constexpr int NC = Packed<DIM>::NC;
 #pragma unroll
     for (int c = 0; c < NC; ++c) lamE[c] = 0.0;
-    for_taps<DIM, STENCIL>(A, u, q, [&](long long p, auto aa, auto kk, TU ua, bool forward, bool lap) {
+    for_taps<DIM, STENCIL, true>(A, u, q, [&](long long p, auto aa, auto kk, TU ua, bool forward, bool lap) {
         constexpr int ax = decltype(aa)::value, k = decltype(kk)::value;
         constexpr double wf = -tap_weight<STENCIL>(true, k), wb = -tap_weight<STENCIL>(false, k);
         double w = Q.g6[ax] * (double)ua * (forward ? wf : wb);
@@ -490,16 +490,18 @@ __device__ __noinline__ void gather_out_of_range(const AdjArgs<double>& A, const
     gather<DIM, STENCIL, float>(A, Q, lamR, u, q, lamE);
 }
 
-// FP64 storage: all in FP64.  FP32 storage (lamR and u hold floats): the FP64 pipe's rate, 1/64 of the FP32
-// pipe's, would bound it (104 operations and as many conversions per 3D point), so weights and sums are
-// three floats each, to more than the accuracy of the FP64 form (largest error of a sum, relative to the sum
-// of its products' magnitudes, 1.1e-16 against 4.3e-16; two floats 2.7e-14).  The weights carry a power of two that
-// keeps the products' rounding errors representable for every normal lamR; sums beyond
-// the float range are formed again in FP64.  Thread = point; the x rows of
-// neighbouring threads come from L1.  3D 64^3, FP32 storage: 60 us, against 92 in FP64 with conversions by integer
-// operations, 140 with the FP64 pipe's, and 33 for sums of two floats.
+// FP64 storage: all in FP64.  FP32 storage (lamR and u hold floats): the FP64 pipe's rate, 1/64 of
+// the FP32 pipe's, would bound it (104 operations and as many conversions per 3D point), so weights
+// and sums are three floats each, to more than the accuracy of the FP64 form (largest error of a
+// sum, relative to the sum of its products' magnitudes, 1.1e-16 against 4.3e-16; two floats
+// 2.7e-14).  The weights carry a power of two that keeps the products' rounding errors
+// representable for every normal lamR; sums beyond the float range are formed again in FP64.  q's
+// own weights of all axes make one product.  Thread = point; the x rows of neighbouring threads
+// come from L1.  3D 64^3, FP32 storage: 50 us (10 blocks per SM; 55 without that bound, 60 with a product per
+// axis for q itself), against 92 in FP64 with conversions by integer operations, 140 with the FP64
+// pipe's, and 33 for sums of two floats.
 template <typename TU, int DIM, int STENCIL>
-__global__ void __launch_bounds__(128) adj_transport_kernel(const AdjArgs<double> A, const GatherScales Q,
+__global__ void __launch_bounds__(128, DIM == 3 ? 10 : 12) adj_transport_kernel(const AdjArgs<double> A, const GatherScales Q,
                                                             const TU* __restrict__ lamR, const TU* __restrict__ u) {
     constexpr int NC = Packed<DIM>::NC;
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -511,25 +513,17 @@ __global__ void __launch_bounds__(128) adj_transport_kernel(const AdjArgs<double
         f3 s[NC];
 #pragma unroll
         for (int c = 0; c < NC; ++c) s[c] = f3{0.0f, 0.0f, 0.0f};
-        for_taps<DIM, STENCIL>(A, u, q, [&](long long p, auto aa, auto kk, float ua, bool forward, bool lap) {
-            constexpr int ax = decltype(aa)::value, k = decltype(kk)::value;
-            constexpr int wf = tap_weight<STENCIL>(true, k), wb = tap_weight<STENCIL>(false, k);
-            // -w6 g6 u [+ lap] as three floats
-            f3 w{0.0f, 0.0f, 0.0f};
-            if constexpr (wf != 0 || wb != 0) {
-                constexpr int mf = wf < 0 ? -wf : wf, mb = wb < 0 ? -wb : wb;
-                const F3c g = (forward ? mf : mb) == mf ? Q.tap[ax][mf] : Q.tap[ax][mb];
-                const float us = (forward ? wf : wb) > 0 ? -ua : ua;
-                const f2 p0 = two_prod(g.a, us), p1 = two_prod(g.b, us);
-                const f2 t = two_sum_f2(p0.lo, p1.hi), h = fast_two_sum(p0.hi, t.hi);
-                w = f3{h.hi, h.lo, __fadd_rn(t.lo, __fmaf_rn(g.c, us, p1.lo))};
-            }
-            if (lap) {
-                const F3c l = Q.lapf[ax][k == 0 ? 1 : 0];
-                w.add(l.a);
-                w.add_small(l.b);
-                w.c = __fadd_rn(w.c, l.c);
-            }
+        auto product = [](const F3c& g, float v) {   // g v
+            const f2 p0 = two_prod(g.a, v), p1 = two_prod(g.b, v);
+            const f2 t = two_sum_f2(p0.lo, p1.hi), h = fast_two_sum(p0.hi, t.hi);
+            return f3{h.hi, h.lo, __fadd_rn(t.lo, __fmaf_rn(g.c, v, p1.lo))};
+        };
+        auto join = [](f3& w, const auto& v) {
+            w.add(v.a);
+            w.add_small(v.b);
+            w.c = __fadd_rn(w.c, v.c);
+        };
+        auto apply = [&](const f3& w, long long p) {
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 const float v = __ldg(lamR + (long long)c * A.N + p);
@@ -539,6 +533,22 @@ __global__ void __launch_bounds__(128) adj_transport_kernel(const AdjArgs<double
                 s[c].add_small(a1.hi);
                 s[c].c = __fadd_rn(s[c].c, __fmaf_rn(w.c, v, a1.lo));
             }
+        };
+        // weights: -w6 g6 u [+ lap]; q's own, of all axes, at once
+        f3 own{0.0f, 0.0f, 0.0f};
+        static_for<0, DIM>([&](auto aa) {
+            constexpr int ax = decltype(aa)::value;
+            if constexpr (STENCIL == 0) join(own, product(Q.tap[ax][3], -fabsf(__ldg(u + (long long)ax * A.N + q))));
+            if (A.eps != 0.0) join(own, Q.lapf[ax][1]);
+        });
+        if (own.a != 0.0f) apply(own, q);
+        for_taps<DIM, STENCIL, false>(A, u, q, [&](long long p, auto aa, auto kk, float ua, bool forward, bool lap) {
+            constexpr int ax = decltype(aa)::value, k = decltype(kk)::value;
+            constexpr int wf = tap_weight<STENCIL>(true, k), wb = tap_weight<STENCIL>(false, k);
+            constexpr int mf = wf < 0 ? -wf : wf, mb = wb < 0 ? -wb : wb;
+            f3 w = product((forward ? mf : mb) == mf ? Q.tap[ax][mf] : Q.tap[ax][mb], (forward ? wf : wb) > 0 ? -ua : ua);
+            if (lap) join(w, Q.lapf[ax][0]);
+            apply(w, p);
         });
         bool finite = true;
 #pragma unroll

@@ -355,9 +355,11 @@ __device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
 
 // A sum of floats to at least the accuracy of FP64 additions, off the FP64 pipe
 // (1/64 of the FP32 rate): the errors of the first float's additions, exact by TwoSum, are
-// summed in a second, and those of the second's in a third (72 bits; sums do not underflow).
+// summed in a second, and those of the second's in a third (72 bits; sums do not underflow; the owner
+// moves a sum that is large() to FP64 before the next addition could leave the float range).
 struct f3 {
     float a, b, c;
+    __device__ __forceinline__ bool large() const { return fabsf(a) > 1.2676506e30f; }   // 2^100
     __device__ __forceinline__ void add(float v) {
         const f2 t = two_sum_f2(a, v);
         a = t.hi;
@@ -373,8 +375,14 @@ struct f3 {
     __device__ __forceinline__ void value(double& hi, double& lo) const {
         hi = (double)a + (double)b;
         lo = ((double)a - hi) + (double)b + (double)c;   // |a| >= |b|
+        if (!isfinite(a)) {   // a alone follows the additions of infinities and NaN
+            hi = (double)a;
+            lo = 0.0;
+        }
     }
-    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+    __device__ __forceinline__ double value() const {
+        return isfinite(a) ? (double)a + ((double)b + (double)c) : (double)a;
+    }
 };
 
 // ----------------------------------------------------------- FP32 point solve

@@ -10,7 +10,7 @@
 // adjoint of a right-hand side is bitwise the one that stepping gives.  The gradients are
 // their sums over the steps, which stepping adds up in FP64 and a run in three floats
 // (no less accurate; the FP64 additions took 4.8 us per reverse step at 2D 512^2, these
-// 1 us more than two floats).  Per step a tile of 32
+// 1.5 us more than two floats).  Per step a tile of 32
 // points exchanges only its right-hand sides and solutions through shared
 // memory; the point matrix is factored once.
 //
@@ -20,7 +20,7 @@
 // tile, which rotates with the tile so that the solves spread over the SM's
 // schedulers.  Nothing but one stress row per step and, per launch, the mode levels moves:
 // a single step is bound by 3 words per (mode, component) from HBM.  Measured at 2D
-// 512^2, m = 32, 100 steps: 15.7 us per step against 49 for tfs_step, 14.1 us per
+// 512^2, m = 32, 100 steps: 15.7 us per step against 49 for tfs_step, 14.6 us per
 // reverse step against 77; a training pass (forward and gradients) 19.2 -> 3.5 ms, of which
 // 4.9 ms are the segments' recomputation that stored stresses make unnecessary.
 // Tried and not kept: one mode sweep per block of eight steps with the steps' own drives convolved
@@ -235,6 +235,19 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
     double sig_sum = 0.0, sym_sum = 0.0;
 #pragma unroll
     for (int e = 0; e < kPer; ++e) gk[e] = f3{0.0f, 0.0f, 0.0f};
+    // to the FP64 fields: the sum of eta lamR - S, and of dJ/dkappa's entries
+    auto flush = [&] {
+        double lh, ll, sh, sl;
+        l_sum.value(lh, ll);
+        s_sum.value(sh, sl);
+        if (active) A.g_sigma0[(long long)c * N + p] += fma(A.eta, lh, -sh) + fma(A.eta, ll, -sl);
+        l_sum = s_sum = f3{0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            if (c + e * NC < DD && active) A.g_kap[(long long)(c + e * NC) * N + p] += gk[e].value();
+            gk[e] = f3{0.0f, 0.0f, 0.0f};
+        }
+    };
 #pragma unroll 1
     for (int k = 0; k < A.steps; ++k) {
         const int n = A.steps - 1 - k;
@@ -285,6 +298,7 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
             s_sum.add(ss);
             s_sum.add_small(-comp);
         }
+        bool large = l_sum.large() | s_sum.large();
         // dJ/dkappa_ab += dt sum_s Lam_as sigma_bs + dt G g Lam_ab, Lam symmetric with doubled diagonal
 #pragma unroll
         for (int e = 0; e < kPer; ++e) {
@@ -292,16 +306,19 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
             if (q < DD) {
                 const int a = q / DIM, b = q % DIM;
                 auto at = [&](int i, int j) { return i == j ? (DIM == 2 ? 2 * i : i) : (DIM == 2 ? 1 : 6 - i - j); };
-                float g = 0.0f;
+                // (dt lamR before sigma: their product may leave the float range where dt times it does not)
+                const float lab = sL[at(a, b)][lane];
+                float g = A.src[k] * (a == b ? 2.0f * lab : lab);
 #pragma unroll
                 for (int s = 0; s < DIM; ++s) {
-                    const float la = sL[at(a, s)][lane];
+                    const float la = A.dt * sL[at(a, s)][lane];
                     g = __fmaf_rn(a == s ? 2.0f * la : la, sSig[k & 1][at(b, s)][lane], g);
                 }
-                const float lab = sL[at(a, b)][lane];
-                gk[e].add(__fmaf_rn(A.dt, g, A.src[k] * (a == b ? 2.0f * lab : lab)));
+                gk[e].add(g);
+                large |= gk[e].large();
             }
         }
+        if (large) flush();
     }
     if (active) {
         if (fl) atomicOr(A.flags, fl);
@@ -310,14 +327,7 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
             __stcs(A.ell_prev + base + j * row, x[j]);
             __stcs(A.ell_prev2 + base + j * row, y[j]);
         });
-        // sum of eta lamR - S over the steps
-        double lh, ll, sh, sl;
-        l_sum.value(lh, ll);
-        s_sum.value(sh, sl);
-        A.g_sigma0[(long long)c * N + p] += fma(A.eta, lh, -sh) + fma(A.eta, ll, -sl);
-#pragma unroll
-        for (int e = 0; e < kPer; ++e)
-            if (c + e * NC < DD) A.g_kap[(long long)(c + e * NC) * N + p] += gk[e].value();
+        flush();
     }
     if (c == ws) {
         const double sd = active ? sig_sum : 0.0, sy = active ? sym_sum : 0.0;

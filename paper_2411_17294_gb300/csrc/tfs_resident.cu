@@ -106,9 +106,12 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_run_kernel(const
     const int ci = Packed<DIM>::I(c), cj = Packed<DIM>::J(c);
     const float s0 = A.sigma0 ? __ldg(A.sigma0 + (long long)c * N + pc) : 0.0f;
     sS0[c][lane] = s0;
-    // kappa* = 2 kappa - kappa = kappa exactly
-    const f2 ks = f2_add(f2{__ldg(A.kap + (long long)(ci * DIM + cj) * N + pc), 0.0f},
-                         f2{__ldg(A.kap + (long long)(cj * DIM + ci) * N + pc), 0.0f});
+    // kappa* = 2 kappa - kappa as the step forms it: kappa exactly, and a NaN from an infinite one
+    auto star = [&](int e) {
+        const float v = __ldg(A.kap + (long long)e * N + pc);
+        return two_sum_f2(2.0f * v, -v);
+    };
+    const f2 ks = f2_add(star(ci * DIM + cj), star(cj * DIM + ci));
     const f2 es0 = f2_mul_f(f2{A.eta.hi, A.eta.lo}, s0);
     unsigned fl = 0u;
     if (c == ws) {
@@ -117,9 +120,8 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_run_kernel(const
         for (int i = 0; i < DIM; ++i)
 #pragma unroll
             for (int j = 0; j < DIM; ++j) {
-                const float v = __ldg(A.kap + (long long)(i * DIM + j) * N + pc);
-                K[i][j] = f2{v, 0.0f};
-                sK[i * DIM + j][lane] = v;
+                K[i][j] = star(i * DIM + j);
+                sK[i * DIM + j][lane] = K[i][j].hi;
             }
         LU32<NC> F;
         if (!factor_point_f32<DIM>(K, A.a, A.dt, F)) fl |= 2u;
@@ -215,7 +217,8 @@ __global__ void __launch_bounds__(kT* Packed<DIM>::NC) resident_back_kernel(cons
         for (int i = 0; i < DIM; ++i)
 #pragma unroll
             for (int j = 0; j < DIM; ++j) {
-                K[i][j] = __ldg(A.kap + (long long)(i * DIM + j) * N + pc);
+                const float v = __ldg(A.kap + (long long)(i * DIM + j) * N + pc);
+                K[i][j] = __fmaf_rn(2.0f, v, -v);   // kappa* (a NaN from an infinite kappa)
                 sK[i * DIM + j][lane] = K[i][j];
             }
         LU32<NC> F;
